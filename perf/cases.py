@@ -318,7 +318,7 @@ def work(case):
     kind = case["kind"]
     if kind == "serve":
         b = f = 0
-        for c in [dict(n=90, views=80, events=480_000)] * case["systems"]:
+        for c in _serve_cases(case):
             b += case["iters"] * (16 * c["events"]) + 4 * (_rows(c) + c["n"] ** 3)
             f += case["iters"] * 4 * c["events"]
         return dict(bytes=b, flops=f)
