@@ -329,11 +329,12 @@ static int finish_system(mc_system *sys, cudaStream_t s) {
   return MC_OK;
 }
 
-constexpr int kCounters = 7;  // events, fates[4], queue fill, largest queue fill
+constexpr int kCounters = 8;  // events, fates[4], queue fill, largest queue fill, histories taken
 
 __global__ void queue_reset_kernel(unsigned long long *ctr) {
   if (ctr[5] > ctr[6]) ctr[6] = ctr[5];
   ctr[5] = 0ull;
+  ctr[7] = 0ull;
 }
 
 // Result of the transport + detection part of a build (the tally, before
@@ -411,6 +412,7 @@ static int tally_from_plan(mc_plan *pl, uint64_t first, uint64_t count, uint64_t
     ts.esc = esc.p;
     ts.esc_capacity = cap_q;
     ts.esc_cursor = ctr.as<unsigned long long>() + 5;
+    ts.work = ctr.as<unsigned long long>() + 7;
     ts.records = nullptr;
     ts.weights = weighted ? out.weights.as<unsigned long long>() : nullptr;
     for (uint64_t c = 0; c < n_chunks; ++c) {

@@ -207,6 +207,7 @@ struct TransportSetup {
   void *esc;                   // escape queue (EscapeRec of the precision)
   unsigned long long esc_capacity;
   unsigned long long *esc_cursor;
+  unsigned long long *work;    // next history a warp takes (analog float path; 0 at the launch)
   cudaEvent_t ev_mid;          // recorded between transport and detection (optional)
   int precision;
   int primary_only;            // tally only unscattered photons

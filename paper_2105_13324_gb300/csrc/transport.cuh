@@ -1,8 +1,12 @@
-// transport.cuh -- persistent photon-history kernel (paper Sec. 2: follow
+// transport.cuh -- photon-history kernels (paper Sec. 2: follow
 // each source photon until it is absorbed, leaves the energy window or
 // escapes, sampling every step from the cross-sections; Sec. 3: parallel-hole
 // collimation and the detection window; Sec. 5.1: the detections estimate the
 // response matrix T_ij of Eq. (IMC)).
+//
+// The analog production builds (float) run histories.cuh's kernel; the kernels
+// here are the double path, the per-history traces, forced detection and the
+// detection of queued escapes.
 //
 // Included by transport_f32.cu (production, float) and transport_f64.cu
 // (verification, double, compiled with --fmad=false so that every product and
@@ -80,6 +84,10 @@ template <typename T> struct TArgs {
   int forced_dir;                   // forced emission direction: cos(theta) in (-band, band)
   T band;                           // sin of the acceptance half-angle
   unsigned long long q_dir;         // fixed-point weight of a detection under forced direction
+  unsigned long long *work;         // history_kernel: next history not yet taken by a warp
+  uint32_t grab;                    // ... histories a warp takes at a time (a multiple of 32)
+  uint32_t first_v;                 // ... first mod N
+  uint32_t magic_n, magic_xy, magic_x;  // ... floor(2^32 / d) of N, nx ny, nx (div_magic)
 };
 
 // An escaping photon that may pass a collimator: its history, the position
@@ -313,28 +321,32 @@ template <typename T> __device__ __forceinline__ int voxel_index(T x, T half, T 
 // Compton scatter by rejection: mu uniform in [-1,1], eps = 1/(1 + a(1-mu)),
 // accepted with probability eps^2 (eps + 1/eps - (1 - mu^2)) / 2 (the
 // Klein-Nishina density over its maximum).
-template <typename T, typename R>
-__device__ __forceinline__ bool compton(R &rng, T e, T &mu_out, T &eps_out) {
+template <typename T>
+__device__ __forceinline__ bool compton_trial(T e, uint32_t w_mu, uint32_t w_acc, T &mu_out, T &eps_out) {
   T alpha;
   if constexpr (is_dbl<T>()) alpha = e / kMec2;
   else alpha = e * (float)(1.0 / kMec2);
+  const T mu = (T)2 * uniform<T>(w_mu) - (T)1;
+  const T den = (T)1 + alpha * ((T)1 - mu);
+  T eps, f;
+  if constexpr (is_dbl<T>()) {
+    eps = 1.0 / den;
+    f = 0.5 * eps * eps * (eps + 1.0 / eps - (1.0 - mu * mu));
+  } else {
+    eps = __fdividef(1.0f, den);
+    // mu^2 rounded on its own, as in rotate(): the same decision in every kernel
+    f = 0.5f * eps * eps * (eps + den - __fsub_rn(1.0f, __fmul_rn(mu, mu)));
+  }
+  mu_out = mu;
+  eps_out = eps;
+  return uniform<T>(w_acc) < f;
+}
+template <typename T, typename R>
+__device__ __forceinline__ bool compton(R &rng, T e, T &mu_out, T &eps_out) {
   for (uint32_t t = 0; t < kTrialCap; ++t) {
     rng.need(2);
-    const T mu = (T)2 * uniform<T>(rng.next()) - (T)1;
-    const T den = (T)1 + alpha * ((T)1 - mu);
-    T eps, f;
-    if constexpr (is_dbl<T>()) {
-      eps = 1.0 / den;
-      f = 0.5 * eps * eps * (eps + 1.0 / eps - (1.0 - mu * mu));
-    } else {
-      eps = __fdividef(1.0f, den);
-      f = 0.5f * eps * eps * (eps + den - (1.0f - mu * mu));
-    }
-    if (uniform<T>(rng.next()) < f) {
-      mu_out = mu;
-      eps_out = eps;
-      return true;
-    }
+    const uint32_t w_mu = rng.next(), w_acc = rng.next();
+    if (compton_trial<T>(e, w_mu, w_acc, mu_out, eps_out)) return true;
   }
   return false;
 }
@@ -359,7 +371,10 @@ template <typename T> __device__ __forceinline__ void rotate(T &u, T &v, T &w, T
     v = nv / n;
     w = nw / n;
   } else {
-    const float st = sqrt0<float>(1.0f - mu * mu);
+    // mu^2 rounded before the subtraction, so that every kernel that calls
+    // this turns a photon by the same bits (a contraction here differs in the
+    // last place, which moves a handful of detections per 10^9 histories)
+    const float st = sqrt0<float>(__fsub_rn(1.0f, __fmul_rn(mu, mu)));
     float nu, nv, nw;
     if (fabsf(w) < 0.99999f) {
       const float r2 = 1.0f - w * w;
@@ -1213,6 +1228,12 @@ template <typename T> void make_targs(const TransportSetup &ts, TArgs<T> &a) {
   a.esc_capacity = ts.esc_capacity;
   a.esc_cursor = ts.esc_cursor;
   a.weights = ts.weights;
+  a.work = ts.work;
+  a.first_v = (uint32_t)(ts.first % a.n_vox);
+  const auto magic = [](uint32_t d) { return d <= 1u ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d); };
+  a.magic_n = magic(a.n_vox);
+  a.magic_xy = magic((uint32_t)ts.nx * (uint32_t)ts.ny);
+  a.magic_x = magic((uint32_t)ts.nx);
   const double cos_max = 1.0 / std::sqrt(1.0 + tan_max * tan_max);
   const double omega = 2.0 * kPi * (1.0 - cos_max);
   a.cos_max = (T)cos_max;
@@ -1239,7 +1260,7 @@ template <typename T> int launch_transport_t(const TransportSetup &ts, cudaStrea
     MCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, transport_kernel<T, false, true>, threads, 0));
   } else if (ts.records) {
     MCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, transport_kernel<T, true>, threads, 0));
-  } else {
+  } else if constexpr (is_dbl<T>()) {  // analog float builds: histories.cuh
     MCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, transport_kernel<T, false>, threads, 0));
   }
   if (per_sm < 1) per_sm = 1;
@@ -1255,13 +1276,13 @@ template <typename T> int launch_transport_t(const TransportSetup &ts, cudaStrea
   }
   if (ts.forced) { count_launch(); transport_kernel<T, false, true><<<grid, threads, 0, s>>>(a); }
   else if (ts.records) { count_launch(); transport_kernel<T, true><<<grid, threads, 0, s>>>(a); }
-  else { count_launch(); transport_kernel<T, false><<<grid, threads, 0, s>>>(a); }
+  else if constexpr (is_dbl<T>()) { count_launch(); transport_kernel<T, false><<<grid, threads, 0, s>>>(a); }
   MCS_LAUNCHED();
   if (ts.ev_mid) MCS_CUDA(cudaEventRecord(ts.ev_mid, s));
   const int dgrid = device_sm_count() * 8;
   if (ts.forced) { count_launch(); fd_kernel<T><<<dgrid, 256, 0, s>>>(a); }
   else if (ts.records) { count_launch(); detect_kernel<T, true><<<dgrid, 256, 0, s>>>(a); }
-  else { count_launch(); detect_kernel<T, false><<<dgrid, 256, 0, s>>>(a); }
+  else if constexpr (is_dbl<T>()) { count_launch(); detect_kernel<T, false><<<dgrid, 256, 0, s>>>(a); }
   MCS_LAUNCHED();
   return MC_OK;
 }

@@ -1,6 +1,7 @@
-// transport_f32.cu -- production (float) instantiation of the photon-history
-// kernel; see transport.cuh.
-#include "transport.cuh"
+// transport_f32.cu -- production (float) transport: the analog photon-history
+// kernel of histories.cuh, and transport.cuh's float instantiations (forced
+// detection, per-history traces).
+#include "histories.cuh"
 
 namespace mcs {
 void compute_coefficients(const TransportSetup &ts, std::vector<double> &cd, std::vector<float> &cf,
@@ -8,7 +9,9 @@ void compute_coefficients(const TransportSetup &ts, std::vector<double> &cd, std
   host_coefficients(ts, cd, cf);
   host_sigma_table(ts, sig_tab);
 }
-int launch_transport_f32(const TransportSetup &ts, cudaStream_t s) { return launch_transport_t<float>(ts, s); }
+int launch_transport_f32(const TransportSetup &ts, cudaStream_t s) {
+  return ts.forced || ts.records ? launch_transport_t<float>(ts, s) : launch_histories(ts, s);
+}
 int launch_debug_kn_f32(double e, uint64_t seed, uint64_t n, double *c, double *p, cudaStream_t s) {
   return launch_debug_kn_t<float>(e, seed, n, c, p, s);
 }
