@@ -383,7 +383,9 @@ static int tally_from_plan(mc_plan *pl, uint64_t first, uint64_t count, uint64_t
   const uint64_t n_chunks = (count + kChunk - 1) / kChunk;
   const uint64_t chunk_max = count < kChunk ? count : kChunk;
   const double acc = tan_max * tan_max / 16.0;
-  double est = forced ? (double)count * (double)ts.n_views * 2.0 + 65536.0
+  // (Forced: about half of 2.2 events per history and view come; assembly
+  // reuses the two buffers for 16-byte entries on their way to the CSR.)
+  double est = forced ? (double)count * (double)ts.n_views * 2.2 + 65536.0
                       : (double)count * (double)ts.n_views * acc * 1.25 / (ts.forced_dir ? band : 1.0) + 65536.0;
   if (est > 4.0e9) est = 4.0e9;
   double est_q = forced ? (double)chunk_max * 3.0 + 65536.0
@@ -488,7 +490,7 @@ static int build_from_plan(mc_plan *pl, uint64_t first, uint64_t count, uint64_t
   cudaEventRecord(e0, s);
   sys->n_events = (int64_t)t.hctr[0];
   for (int f = 0; f < 4; ++f) sys->fates[f] = t.hctr[1 + f];
-  rc = assemble_system(sys, t.events, sys->n_events, s, weighted ? t.weights.as<uint64_t>() : nullptr);
+  rc = assemble_system(sys, t.events, sys->n_events, s, weighted ? &t.weights : nullptr);
   if (rc == MC_OK) {
     t.weights.release();
     rc = finish_system(sys, s);
@@ -864,7 +866,7 @@ int mc_system_from_weighted_events(int64_t n_rows, int64_t n_cols, const int32_t
   }
   r.release();
   c.release();
-  if ((rc = assemble_system(sys, keys, n_events, s, w.as<uint64_t>()))) return fail(rc);
+  if ((rc = assemble_system(sys, keys, n_events, s, &w))) return fail(rc);
   w.release();
   if ((rc = finish_system(sys, s))) return fail(rc);
   *out = sys;

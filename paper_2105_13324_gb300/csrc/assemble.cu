@@ -463,6 +463,15 @@ static int bits_for(uint64_t range) {
   return b;
 }
 
+// Quotient of a key by a fixed divisor: the estimate by floor((2^64 - 1) / m)
+// is the true quotient or one less.
+struct Div64 { uint64_t m, magic; };
+static Div64 make_div(uint64_t m) { return Div64{m, ~0ull / m}; }
+__device__ __forceinline__ uint64_t div_key(uint64_t k, const Div64 &d) {
+  const uint64_t q = __umul64hi(k, d.magic);
+  return k - q * d.m >= d.m ? q + 1 : q;
+}
+
 // ---------------------------------------------------------------------------
 // assembly by buckets (unweighted events, short columns and rows)
 // ---------------------------------------------------------------------------
@@ -475,19 +484,19 @@ static int bits_for(uint64_t range) {
 // than kBucketLen events and no row more than kBucketLen entries.
 constexpr int kBucketLen = 64;
 
-__global__ void bucket_count_kernel(const uint64_t *keys, int64_t n, uint64_t m, uint32_t *cnt) {
+__global__ void bucket_count_kernel(const uint64_t *keys, int64_t n, Div64 m, uint32_t *cnt) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&cnt[keys[i] / m], 1u);
+    atomicAdd(&cnt[div_key(keys[i], m)], 1u);
 }
 
 // event i -> its row, at start[column] + (its place among the column's
 // events, in arrival order at the atomic)
-__global__ void bucket_fill_kernel(const uint64_t *keys, int64_t n, uint64_t m, const uint32_t *start,
+__global__ void bucket_fill_kernel(const uint64_t *keys, int64_t n, Div64 m, const uint32_t *start,
                                    uint32_t *cursor, uint32_t *minor) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t k = keys[i];
-    const uint64_t v = k / m;
-    minor[start[v] + atomicAdd(&cursor[v], 1u)] = (uint32_t)(k - v * m);
+    const uint64_t v = div_key(k, m);
+    minor[start[v] + atomicAdd(&cursor[v], 1u)] = (uint32_t)(k - v * m.m);
   }
 }
 
@@ -637,13 +646,14 @@ __global__ void transpose_fill_kernel(const uint32_t *col_ptr, int64_t n_cols, c
 static int assemble_buckets(mc_system *sys, const uint64_t *keys, int64_t n, cudaStream_t s, bool *done) {
   *done = false;
   const int64_t M = sys->n_rows, N = sys->n_cols;
+  const Div64 dm = make_div((uint64_t)M);
   DevBuf ccnt, start, flag;
   MCS_TRY(ccnt.alloc((size_t)(N + 1) * sizeof(uint32_t), s));
   MCS_TRY(start.alloc((size_t)(N + 1) * sizeof(uint32_t), s));
   MCS_TRY(flag.alloc(sizeof(unsigned int), s));
   MCS_CUDA(cudaMemsetAsync(ccnt.p, 0, (size_t)(N + 1) * sizeof(uint32_t), s));
   MCS_CUDA(cudaMemsetAsync(flag.p, 0, sizeof(unsigned int), s));
-  count_launch(); bucket_count_kernel<<<grid_for(n), 256, 0, s>>>(keys, n, (uint64_t)M, ccnt.as<uint32_t>());
+  count_launch(); bucket_count_kernel<<<grid_for(n), 256, 0, s>>>(keys, n, dm, ccnt.as<uint32_t>());
   MCS_LAUNCHED();
   MCS_TRY(exclusive_scan_u32(ccnt.as<uint32_t>(), start.as<uint32_t>(), N + 1, s));
   // events into column buckets, sorted and merged
@@ -652,7 +662,7 @@ static int assemble_buckets(mc_system *sys, const uint64_t *keys, int64_t n, cud
   MCS_TRY(ecnt.alloc((size_t)n * sizeof(uint32_t), s));
   MCS_CUDA(cudaMemsetAsync(ccnt.p, 0, (size_t)(N + 1) * sizeof(uint32_t), s));  // now the bucket cursors
   count_launch();
-  bucket_fill_kernel<<<grid_for(n), 256, 0, s>>>(keys, n, (uint64_t)M, start.as<uint32_t>(), ccnt.as<uint32_t>(),
+  bucket_fill_kernel<<<grid_for(n), 256, 0, s>>>(keys, n, dm, start.as<uint32_t>(), ccnt.as<uint32_t>(),
                                                  minor.as<uint32_t>());
   MCS_LAUNCHED();
   // ccnt becomes the merged entries per column (ccnt[N] stays 0 for the scan)
@@ -707,6 +717,636 @@ static int assemble_buckets(mc_system *sys, const uint64_t *keys, int64_t n, cud
   MCS_CUDA(cudaStreamSynchronize(s));
   if (too_long) return MC_OK;  // a row of more than kBucketLen entries
   sys->nnz = nnz;
+  *done = true;
+  return MC_OK;
+}
+
+// ---------------------------------------------------------------------------
+// assembly by sorted segments (weighted events, and columns or rows too long
+// for the buckets above)
+// ---------------------------------------------------------------------------
+// The events are placed in their columns' segments as above; a warp then
+// sorts each column by row in its registers, counts the distinct rows, and,
+// once the column pointers are known, sorts again and writes the merged
+// entries, their projector values and the column sums.  The CSR is made the
+// same way: entries placed in their rows' segments, a warp per row.  Sorting
+// twice (~2 warp instructions per event) is cheaper than writing the sorted
+// events out and reading them back.  Integer work on whole segments, so the
+// matrix does not depend on the order of arrival.
+//
+// Bound by the placement passes (a scattered store per entry, and a returning
+// atomic per run of events of one column) and by memory otherwise: about 110
+// bytes a weighted event in all against ~310 for the radix sort's nine passes
+// and its gather.  2.6e8 weighted events of a forced-detection build: 38.3 ->
+// 18.3 ms; 7.3e7 counted events in columns of ~35 (which the buckets tried
+// first, in vain): 14.4 -> 6.7 ms, with its first projections.
+constexpr int kSegLen = 1024;  // longest segment: 32 elements per lane
+// Segments of up to 256 elements and longer ones are two launches of each
+// kernel: with 8 keys a lane instead of 32 an SM holds twice the warps.
+constexpr int kShortK = 8;
+constexpr int kRowBlocks = 1024;  // row blocks of the two-pass transpose, at most
+
+__device__ __forceinline__ uint32_t key_min(uint32_t a, uint32_t b) { return min(a, b); }
+__device__ __forceinline__ uint32_t key_max(uint32_t a, uint32_t b) { return max(a, b); }
+__device__ __forceinline__ uint64_t key_min(uint64_t a, uint64_t b) { return a < b ? a : b; }
+__device__ __forceinline__ uint64_t key_max(uint64_t a, uint64_t b) { return a < b ? b : a; }
+
+// Ascending bitonic sort of 32 K keys over a warp, element lane K + k in
+// r[k].  Each merge starts with a comparison against the mirrored position,
+// so that every comparison puts the smaller key first.  Blocked order keeps
+// all but 15 of the stages inside the lanes.
+template <int K, typename Key> __device__ __forceinline__ void warp_sort(Key (&r)[K], int lane) {
+#pragma unroll
+  for (int size = 2; size <= K; size <<= 1) {
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const int j = i ^ (size - 1);
+      if (j > i) { const Key a = key_min(r[i], r[j]), b = key_max(r[i], r[j]); r[i] = a; r[j] = b; }
+    }
+#pragma unroll
+    for (int d = size / 4; d > 0; d >>= 1)
+#pragma unroll
+      for (int i = 0; i < K; ++i)
+        if (!(i & d)) { const Key a = key_min(r[i], r[i + d]), b = key_max(r[i], r[i + d]); r[i] = a; r[i + d] = b; }
+  }
+#pragma unroll
+  for (int lanes = 2; lanes <= 32; lanes <<= 1) {
+    Key o[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) o[k] = __shfl_xor_sync(0xffffffffu, r[K - 1 - k], lanes - 1);
+    const bool low0 = !(lane & (lanes >> 1));
+#pragma unroll
+    for (int k = 0; k < K; ++k) r[k] = low0 ? key_min(r[k], o[k]) : key_max(r[k], o[k]);
+#pragma unroll
+    for (int d = lanes / 4; d > 0; d >>= 1) {
+      const bool low = !(lane & d);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const Key x = __shfl_xor_sync(0xffffffffu, r[k], d);
+        r[k] = low ? key_min(r[k], x) : key_max(r[k], x);
+      }
+    }
+#pragma unroll
+    for (int d = K / 2; d > 0; d >>= 1)
+#pragma unroll
+      for (int i = 0; i < K; ++i)
+        if (!(i & d)) { const Key a = key_min(r[i], r[i + d]), b = key_max(r[i], r[i + d]); r[i] = a; r[i + d] = b; }
+  }
+}
+
+// Sort the len <= 32 K keys key(0..len-1), unused places last; with `out`
+// (shared memory, 32 K keys) the sorted keys are left there.  Returns the
+// number of distinct keys >> lb where out is NULL.
+template <int K, typename Key, typename F>
+__device__ __forceinline__ uint32_t sort_segment(uint32_t len, int lb, int lane, Key *out, const F &key) {
+  Key r[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t e = 32u * k + lane;
+    r[k] = e < len ? key(e) : ~(Key)0;
+  }
+  warp_sort<K, Key>(r, lane);
+  if (out) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) out[lane * K + k] = r[k];
+    __syncwarp();
+    return 0u;
+  }
+  Key prev = __shfl_up_sync(0xffffffffu, r[K - 1], 1);
+  uint32_t n = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t e = (uint32_t)(lane * K + k);
+    n += e < len && (e == 0u || (prev >> lb) != (r[k] >> lb)) ? 1u : 0u;
+    prev = r[k];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  return n;
+}
+
+// ... with K the smallest power of two that holds len (MAXK at most)
+template <int MAXK, typename Key, typename F>
+__device__ __forceinline__ uint32_t sort_segment_any(uint32_t len, int lb, int lane, Key *out, const F &key) {
+  if (len <= 32) return sort_segment<1, Key>(len, lb, lane, out, key);
+  if (len <= 64) return sort_segment<2, Key>(len, lb, lane, out, key);
+  if (len <= 128) return sort_segment<4, Key>(len, lb, lane, out, key);
+  if (MAXK <= 8 || len <= 256) return sort_segment<8, Key>(len, lb, lane, out, key);
+  if (len <= 512) return sort_segment<(MAXK > 8 ? 16 : 8), Key>(len, lb, lane, out, key);
+  return sort_segment<MAXK, Key>(len, lb, lane, out, key);
+}
+
+__global__ void max_value_kernel(const uint32_t *v, int64_t n, unsigned int *out) {
+  uint32_t mx = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    mx = max(mx, v[i]);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(out, mx);
+}
+
+// Events per column; neighbouring events of one column (forced detection
+// appends a record's copies together) take one atomic.
+__global__ void segment_count_kernel(const uint64_t *keys, int64_t n, Div64 m, uint32_t *cnt) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+    const bool valid = i0 + lane < n;
+    const uint32_t v = valid ? (uint32_t)div_key(keys[i0 + lane], m) : 0xffffffffu;
+    const uint32_t vp = __shfl_up_sync(0xffffffffu, v, 1);
+    const bool head = lane == 0 || v != vp;
+    const unsigned heads = __ballot_sync(0xffffffffu, head);
+    if (head && valid) {
+      const unsigned later = lane < 31 ? heads >> (lane + 1) : 0u;
+      atomicAdd(&cnt[v], later ? (uint32_t)__ffs(later) : 32u - lane);
+    }
+  }
+}
+
+// Events into their columns' segments: cursor[v] starts at the segment's
+// first place.  Four rounds of a warp are in flight at once (the atomics
+// return a place each).
+template <bool W>
+__global__ void __launch_bounds__(256) segment_fill_kernel(const uint64_t *keys, const uint64_t *weights, int64_t n,
+                                                         Div64 m, uint32_t *cursor, uint32_t *rows, uint64_t *w) {
+  constexpr int U = 4;
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i0 = warp * (32 * U); i0 < n; i0 += n_warps * (32 * U)) {
+    uint32_t row[U], place[U];
+    uint64_t wt[U];
+    int leader[U];
+    bool valid[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + 32 * u + lane;
+      valid[u] = i < n;
+      const uint64_t k = valid[u] ? keys[i] : 0ull;
+      if (W) wt[u] = valid[u] ? weights[i] : 0ull;
+      const uint64_t q = div_key(k, m);
+      row[u] = (uint32_t)(k - q * m.m);
+      const uint32_t v = valid[u] ? (uint32_t)q : 0xffffffffu;
+      const uint32_t vp = __shfl_up_sync(0xffffffffu, v, 1);
+      const bool head = lane == 0 || v != vp;
+      const unsigned heads = __ballot_sync(0xffffffffu, head);
+      leader[u] = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+      place[u] = 0u;
+      if (head && valid[u]) {
+        const unsigned later = lane < 31 ? heads >> (lane + 1) : 0u;
+        place[u] = atomicAdd(&cursor[v], later ? (uint32_t)__ffs(later) : 32u - lane);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t p = __shfl_sync(0xffffffffu, place[u], leader[u]) + (uint32_t)(lane - leader[u]);
+      if (valid[u]) {
+        rows[p] = row[u];
+        if (W) w[p] = wt[u];
+      }
+    }
+  }
+}
+
+constexpr int kSegThreads = 256;
+
+// distinct rows of each column
+template <int MAXK>
+__global__ void __launch_bounds__(kSegThreads) segment_unique_kernel(const uint32_t *start, int64_t n_seg,
+                                                                  uint32_t shortest, const uint32_t *rows,
+                                                                  uint32_t *uniq) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n_warps = ((int64_t)gridDim.x * kSegThreads) >> 5;
+  for (int64_t c = ((int64_t)blockIdx.x * kSegThreads + threadIdx.x) >> 5; c < n_seg; c += n_warps) {
+    const uint32_t b = start[c], len = start[c + 1] - b;
+    if (len < shortest || len > 32u * MAXK) continue;  // another launch's
+    uint32_t u = len;
+    if (len > 1u)
+      u = sort_segment_any<MAXK, uint32_t>(len, 0, lane, nullptr, [&](uint32_t e) { return rows[b + e]; });
+    if (lane == 0) uniq[c] = u;
+  }
+}
+
+// One CSR entry on its way to its row's segment.
+template <bool W> struct SegEntry;
+template <> struct alignas(8) SegEntry<false> { uint32_t col, cnt; };
+template <> struct alignas(16) SegEntry<true> { uint32_t col, cnt; uint64_t w; };
+
+// The merged CSC entries of each column in row order, with their values, the
+// column sums and the number of entries per row.  Weighted: keys hold the
+// event's place in the segment below the row (lb bits).
+template <typename Key, int MAXK, bool W>
+__global__ void __launch_bounds__(kSegThreads) segment_merge_kernel(const uint32_t *start, const uint32_t *col_ptr,
+                                                                 int64_t n_seg, uint32_t shortest, const uint32_t *rows,
+                                                                 const uint64_t *w, int lb, uint32_t *row_idx,
+                                                                 uint32_t *cnt, uint64_t *wq, float *val,
+                                                                 double *colsum, float *inv_colsum,
+                                                                 unsigned int *max_count, uint32_t *row_hist) {
+  extern __shared__ __align__(16) unsigned char seg_smem[];
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  Key *s_key = reinterpret_cast<Key *>(seg_smem) + (threadIdx.x >> 5) * (32 * MAXK);
+  const int64_t n_warps = ((int64_t)gridDim.x * kSegThreads) >> 5;
+  const uint32_t mask_lb = (1u << lb) - 1u;
+  uint32_t mx = 0;
+  for (int64_t c = ((int64_t)blockIdx.x * kSegThreads + threadIdx.x) >> 5; c < n_seg; c += n_warps) {
+    const uint32_t b = start[c], len = start[c + 1] - b;
+    if (len < shortest || len > 32u * MAXK) continue;
+    uint32_t out = col_ptr[c];
+    uint64_t w_lo = 0, w_hi = 0;  // the column's weights, summed exactly
+    if (len > 0u) {
+      sort_segment_any<MAXK, Key>(len, lb, lane, s_key, [&](uint32_t e) {
+        return W ? (Key)(((Key)rows[b + e] << lb) | (Key)e) : (Key)rows[b + e];
+      });
+      for (uint32_t e0 = 0; e0 < len; e0 += 32) {
+        const uint32_t e = e0 + lane;
+        const Key k = e < len ? s_key[e] : (Key)0;
+        const uint32_t row = (uint32_t)(k >> lb);
+        const bool head = e < len && (e == 0u || (uint32_t)(s_key[e - 1] >> lb) != row);
+        const unsigned heads = __ballot_sync(0xffffffffu, head);
+        if (head) {
+          uint32_t n = 1;
+          uint64_t acc = W ? w[b + ((uint32_t)k & mask_lb)] : 0ull;
+          for (uint32_t t = e + 1; t < len && (uint32_t)(s_key[t] >> lb) == row; ++t) {
+            n += 1;
+            if (W) acc += w[b + ((uint32_t)s_key[t] & mask_lb)];
+          }
+          const uint32_t o = out + __popc(heads & lt);
+          row_idx[o] = row;
+          cnt[o] = n;
+          if (W) {
+            wq[o] = acc;
+            val[o] = __ull2float_rn(acc) * (float)(1.0 / kFdScale);
+            w_lo += (uint32_t)acc;
+            w_hi += acc >> 32;
+          } else {
+            val[o] = (float)n;
+          }
+          atomicAdd(&row_hist[row], 1u);
+          mx = max(mx, n);
+        }
+        out += __popc(heads);
+      }
+      __syncwarp();
+    }
+    double sum = (double)len;
+    if (W) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        w_lo += __shfl_xor_sync(0xffffffffu, w_lo, o);
+        w_hi += __shfl_xor_sync(0xffffffffu, w_hi, o);
+      }
+      sum = ((double)w_hi * 4294967296.0 + (double)w_lo) * (1.0 / kFdScale);
+    }
+    if (lane == 0) {
+      colsum[c] = sum;
+      inv_colsum[c] = sum > 0.0 ? (float)(1.0 / sum) : 0.0f;
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0 && mx) atomicMax(max_count, mx);
+}
+
+// CSC entries into their rows' segments (cursor[j] starts at row_ptr[j])
+template <bool W>
+__global__ void __launch_bounds__(kSegThreads) segment_transpose_kernel(const uint32_t *col_ptr, int64_t n_cols,
+                                                                     const uint32_t *row_idx, const uint32_t *cnt,
+                                                                     const uint64_t *wq, uint32_t *cursor,
+                                                                     SegEntry<W> *out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n_warps = ((int64_t)gridDim.x * kSegThreads) >> 5;
+  for (int64_t c = ((int64_t)blockIdx.x * kSegThreads + threadIdx.x) >> 5; c < n_cols; c += n_warps) {
+    const uint32_t e = col_ptr[c + 1];
+#pragma unroll 4
+    for (uint32_t k = col_ptr[c] + lane; k < e; k += 32) {
+      SegEntry<W> x;
+      x.col = (uint32_t)c;
+      x.cnt = cnt[k];
+      if constexpr (W) x.w = wq[k];
+      out[atomicAdd(&cursor[row_idx[k]], 1u)] = x;
+    }
+  }
+}
+
+// The same in two passes, for matrices beyond the L2.  Pass 1 sorts tiles of
+// CSC entries by block of 2^shift rows in shared memory and appends each run
+// to its row block's part of the CSR range; in pass 2 one thread block takes a
+// row block and places its entries in their rows' segments, with cursors in
+// shared memory.  2.5e8 entries of 16 bytes (a forced-detection matrix): 3.4 +
+// 5.7 ms against 11.9 ms for the direct transpose, whose returning global
+// atomics run at 50 G/s at best and whose sectors are written back half full.
+// Pass 2 is bound by its 16-byte stores to random sectors (44 G/s).  An entry
+// on its way holds its row within the block and its count (at most kSegLen:
+// 11 bits) in one word.
+constexpr int kPartThreads = 512;
+constexpr int kPartCntBits = 11;
+constexpr int kBlockRows = 4096;  // rows of a row block at most
+template <bool W> constexpr int part_items() { return W ? 8 : 16; }  // entries per thread
+template <bool W> struct PartSmem {
+  SegEntry<W> item[kPartThreads * part_items<W>()];
+  uint16_t block[kPartThreads * part_items<W>()];
+  uint32_t cnt[kRowBlocks], base[kRowBlocks], warp[32];
+};
+
+// largest i in [lo, hi) with v[i] <= x (v[lo] <= x)
+__device__ __forceinline__ int64_t find_le(const uint32_t *v, int64_t lo, int64_t hi, uint32_t x) {
+  while (hi - lo > 1) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (v[mid] <= x) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+// column of the first entry of each tile, and of the last entry
+__global__ void tile_columns_kernel(const uint32_t *col_ptr, int64_t n_cols, uint32_t nnz, uint32_t tile,
+                                    int64_t n_tiles, uint32_t *first) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t <= n_tiles; t += (int64_t)gridDim.x * blockDim.x)
+    first[t] = (uint32_t)find_le(col_ptr, 0, n_cols + 1, t < n_tiles ? (uint32_t)t * tile : nnz - 1u);
+}
+
+template <bool W>
+__global__ void __launch_bounds__(kPartThreads) partition_rows_kernel(const uint32_t *col_ptr, const uint32_t *tile_col,
+                                                                   uint32_t nnz, const uint32_t *row_idx,
+                                                                   const uint32_t *cnt, const uint64_t *wq, int shift,
+                                                                   uint32_t *cursor, SegEntry<W> *out) {
+  constexpr int I = part_items<W>(), T = kPartThreads * I;
+  extern __shared__ __align__(16) unsigned char seg_smem[];
+  PartSmem<W> &sm = *reinterpret_cast<PartSmem<W> *>(seg_smem);
+  const uint32_t p0 = blockIdx.x * (uint32_t)T;
+  const uint32_t n = min((uint32_t)T, nnz - p0);
+  for (int b = threadIdx.x; b < kRowBlocks; b += kPartThreads) sm.cnt[b] = 0u;
+  __syncthreads();
+  const int64_t c0 = tile_col[blockIdx.x], c1 = tile_col[blockIdx.x + 1];
+  SegEntry<W> x[I];
+  uint32_t place[I];  // block | (place among the tile's entries of the block) << 10
+#pragma unroll
+  for (int k = 0; k < I; ++k) {
+    const uint32_t e = threadIdx.x + k * kPartThreads;
+    place[k] = 0u;
+    if (e < n) {
+      const uint32_t row = row_idx[p0 + e], b = row >> shift;
+      x[k].cnt = ((row - (b << shift)) << kPartCntBits) | cnt[p0 + e];
+      if constexpr (W) x[k].w = wq[p0 + e];
+      x[k].col = (uint32_t)find_le(col_ptr, c0, c1 + 1, p0 + e);
+      place[k] = b | (atomicAdd(&sm.cnt[b], 1u) << 10);
+    }
+  }
+  __syncthreads();
+  // each row block's start in the tile, and its run's place in the output
+  const uint32_t n0 = sm.cnt[2 * threadIdx.x], n1 = sm.cnt[2 * threadIdx.x + 1];
+  uint32_t total;
+  const uint32_t at = block_exclusive_scan(n0 + n1, sm.warp, total);
+  sm.cnt[2 * threadIdx.x] = at;
+  sm.cnt[2 * threadIdx.x + 1] = at + n0;
+  if (n0) sm.base[2 * threadIdx.x] = atomicAdd(&cursor[2 * threadIdx.x], n0) - at;
+  if (n1) sm.base[2 * threadIdx.x + 1] = atomicAdd(&cursor[2 * threadIdx.x + 1], n1) - (at + n0);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < I; ++k) {
+    if (threadIdx.x + k * kPartThreads < n) {
+      const uint32_t b = place[k] & 1023u, p = sm.cnt[b] + (place[k] >> 10);
+      sm.item[p] = x[k];
+      sm.block[p] = (uint16_t)b;
+    }
+  }
+  __syncthreads();
+  for (uint32_t p = threadIdx.x; p < n; p += kPartThreads) out[sm.base[sm.block[p]] + p] = sm.item[p];
+}
+
+// first CSR position of each row block
+__global__ void row_block_starts_kernel(const uint32_t *row_ptr, int64_t n_rows, int shift, uint32_t *starts) {
+  const int64_t r = (int64_t)threadIdx.x << shift;
+  starts[threadIdx.x] = row_ptr[r < n_rows ? r : n_rows];
+}
+
+// Pass 2: row block b = rows [b << shift, (b + 1) << shift), its entries those
+// of its CSR range.  Two blocks of 512 threads per SM: the rows being filled
+// are then ~300 x 2048, whose half-written lines (80 MB) stay in the L2.
+constexpr int kPlaceThreads = 512;
+template <bool W>
+__global__ void __launch_bounds__(kPlaceThreads, 2) place_rows_kernel(const SegEntry<W> *in, const uint32_t *row_ptr,
+                                                                   int shift, int64_t n_rows, SegEntry<W> *out) {
+  __shared__ uint32_t s_cur[kBlockRows];
+  extern __shared__ __align__(16) unsigned char seg_smem[];  // unused: keeps a third block off the SM
+  const int64_t r0 = (int64_t)blockIdx.x << shift;
+  const int n = (int)min((int64_t)1 << shift, n_rows - r0);
+  const uint32_t p0 = row_ptr[r0], p1 = row_ptr[r0 + n];
+  for (int r = threadIdx.x; r < n; r += kPlaceThreads) s_cur[r] = row_ptr[r0 + r];
+  __syncthreads();
+  constexpr int I = 8;
+  for (uint32_t p = p0 + threadIdx.x; p < p1; p += I * kPlaceThreads) {
+    SegEntry<W> x[I];
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+      if (p + k * kPlaceThreads < p1) x[k] = in[p + k * kPlaceThreads];
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+      if (p + k * kPlaceThreads < p1) {
+        const uint32_t pos = atomicAdd(&s_cur[x[k].cnt >> kPartCntBits], 1u);
+        x[k].cnt &= (1u << kPartCntBits) - 1u;
+        out[pos] = x[k];
+      }
+  }
+}
+
+// the CSR entries of each row in column order, with their values
+template <typename Key, int MAXK, bool W>
+__global__ void __launch_bounds__(kSegThreads) segment_rows_kernel(const uint32_t *row_ptr, int64_t n_rows,
+                                                                uint32_t shortest, const SegEntry<W> *ent, int lb, uint32_t *col_idx,
+                                                                uint32_t *cnt, uint64_t *wq, float *val) {
+  extern __shared__ __align__(16) unsigned char seg_smem[];
+  const int lane = threadIdx.x & 31;
+  Key *s_key = reinterpret_cast<Key *>(seg_smem) + (threadIdx.x >> 5) * (32 * MAXK);
+  const int64_t n_warps = ((int64_t)gridDim.x * kSegThreads) >> 5;
+  const uint32_t mask_lb = (1u << lb) - 1u;
+  for (int64_t j = ((int64_t)blockIdx.x * kSegThreads + threadIdx.x) >> 5; j < n_rows; j += n_warps) {
+    const uint32_t b = row_ptr[j], len = row_ptr[j + 1] - b;
+    if (len == 0u || len < shortest || len > 32u * MAXK) continue;
+    sort_segment_any<MAXK, Key>(len, lb, lane, s_key,
+                                [&](uint32_t e) { return (Key)(((Key)ent[b + e].col << lb) | (Key)e); });
+    for (uint32_t e = lane; e < len; e += 32) {
+      const Key k = s_key[e];
+      const SegEntry<W> x = ent[b + ((uint32_t)k & mask_lb)];
+      col_idx[b + e] = x.col;
+      cnt[b + e] = x.cnt;
+      if constexpr (W) {
+        wq[b + e] = x.w;
+        val[b + e] = __ull2float_rn(x.w) * (float)(1.0 / kFdScale);
+      } else {
+        val[b + e] = (float)x.cnt;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+static int max_of(const DevBuf &v, int64_t n, DevBuf &scratch, uint32_t *out, cudaStream_t s) {
+  MCS_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(unsigned int), s));
+  count_launch(); max_value_kernel<<<grid_for(n), 256, 0, s>>>(v.as<uint32_t>(), n, scratch.as<unsigned int>());
+  MCS_LAUNCHED();
+  MCS_CUDA(cudaMemcpyAsync(out, scratch.p, sizeof(*out), cudaMemcpyDeviceToHost, s));
+  MCS_CUDA(cudaStreamSynchronize(s));
+  return MC_OK;
+}
+
+template <typename Kernel, typename... A>
+static int launch_segments(Kernel *k, size_t key_bytes, int maxk, int64_t n_seg, cudaStream_t s, A... args) {
+  const size_t smem = (kSegThreads / 32) * 32 * (size_t)maxk * key_bytes;
+  if (smem > 48 * 1024) MCS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  count_launch();
+  k<<<grid_for(n_seg * 32), kSegThreads, smem, s>>>(args...);
+  MCS_LAUNCHED();
+  return MC_OK;
+}
+
+// The CSC and CSR of n > 0 events (with the projector values and the column
+// sums) by sorted segments.  Sets *done, or leaves the matrix unfinished (and
+// the events untouched) when a column holds more than kSegLen events or a row
+// more than kSegLen entries; the events' buffers are released once they are
+// not needed.
+template <bool W>
+static int assemble_segments(mc_system *sys, DevBuf &key_buf, DevBuf *weight_buf, int64_t n, cudaStream_t s,
+                             bool *done) {
+  *done = false;
+  const uint64_t *keys = key_buf.as<uint64_t>(), *weights = W ? weight_buf->as<uint64_t>() : nullptr;
+  const int64_t M = sys->n_rows, N = sys->n_cols;
+  const Div64 dm = make_div((uint64_t)M);
+  DevBuf cnt, start, flag, tmp;
+  MCS_TRY(cnt.alloc((size_t)(N + 1) * 4, s));
+  MCS_TRY(start.alloc((size_t)(N + 1) * 4, s));
+  MCS_TRY(flag.alloc(sizeof(unsigned int), s));
+  MCS_CUDA(cudaMemsetAsync(cnt.p, 0, (size_t)(N + 1) * 4, s));
+  count_launch(); segment_count_kernel<<<grid_for(n), 256, 0, s>>>(keys, n, dm, cnt.as<uint32_t>());
+  MCS_LAUNCHED();
+  MCS_TRY(exclusive_scan_u32(cnt.as<uint32_t>(), start.as<uint32_t>(), N + 1, s));
+  uint32_t longest = 0;
+  MCS_TRY(max_of(cnt, N, flag, &longest, s));
+  if (longest > (uint32_t)kSegLen) return MC_OK;
+  MCS_TRY(tmp.alloc((size_t)n * (W ? 12 : 4), s));  // weights, then rows
+  uint64_t *const w = W ? tmp.as<uint64_t>() : nullptr;
+  uint32_t *const rows = reinterpret_cast<uint32_t *>(tmp.as<uint64_t>() + (W ? n : 0));
+  MCS_CUDA(cudaMemcpyAsync(cnt.p, start.p, (size_t)(N + 1) * 4, cudaMemcpyDeviceToDevice, s));  // now the cursors
+  count_launch();
+  segment_fill_kernel<W><<<grid_for((n + 3) / 4), 256, 0, s>>>(keys, weights, n, dm, cnt.as<uint32_t>(),
+                                                               rows, w);
+  MCS_LAUNCHED();
+  // distinct rows per column, column pointers
+  MCS_CUDA(cudaMemsetAsync(cnt.as<uint32_t>() + N, 0, 4, s));
+  MCS_TRY(launch_segments(segment_unique_kernel<kShortK>, 0, 1, N, s, start.as<uint32_t>(), N, 0u, rows,
+                          cnt.as<uint32_t>()));
+  if (longest > 32 * kShortK)
+    MCS_TRY(launch_segments(segment_unique_kernel<32>, 0, 1, N, s, start.as<uint32_t>(), N, 32u * kShortK + 1u,
+                            rows, cnt.as<uint32_t>()));
+  MCS_TRY(sys->col_ptr.alloc((size_t)(N + 1) * 4, s));
+  MCS_TRY(exclusive_scan_u32(cnt.as<uint32_t>(), sys->col_ptr.as<uint32_t>(), N + 1, s));
+  uint32_t nnz = 0;
+  MCS_CUDA(cudaMemcpyAsync(&nnz, sys->col_ptr.as<uint32_t>() + N, sizeof(nnz), cudaMemcpyDeviceToHost, s));
+  MCS_CUDA(cudaStreamSynchronize(s));
+  // CSC entries
+  DevBuf rhist;
+  MCS_TRY(sys->row_idx.alloc((size_t)nnz * 4, s));
+  MCS_TRY(sys->csc_cnt.alloc((size_t)nnz * 4, s));
+  MCS_TRY(sys->csc_val.alloc((size_t)nnz * 4, s));
+  if (W) MCS_TRY(sys->csc_wq.alloc((size_t)nnz * 8, s));
+  MCS_TRY(sys->colsum.alloc((size_t)N * sizeof(double), s));
+  MCS_TRY(sys->inv_colsum.alloc((size_t)N * sizeof(float), s));
+  // two-pass transpose from 256 MB of entries on (below, the direct one's
+  // scattered stores stay in the L2), in up to kRowBlocks blocks of rows
+  int shift = 0;
+  if ((uint64_t)nnz * sizeof(SegEntry<W>) > (256ull << 20) && M > kRowBlocks && M <= (int64_t)kRowBlocks * kBlockRows)
+    while (((M - 1) >> shift) + 1 > kRowBlocks) ++shift;
+  MCS_TRY(rhist.alloc((size_t)(M + 1) * 4, s));
+  MCS_CUDA(cudaMemsetAsync(rhist.p, 0, (size_t)(M + 1) * 4, s));
+  MCS_CUDA(cudaMemsetAsync(flag.p, 0, sizeof(unsigned int), s));
+  {
+    const int lb = W ? bits_for(longest - 1) : 0;
+    const bool wide = W && bits_for((uint64_t)M - 1) + lb > 32;
+    auto go = [&](auto *k, size_t kb, int maxk) {
+      return launch_segments(k, kb, maxk, N, s, (const uint32_t *)start.as<uint32_t>(),
+                             (const uint32_t *)sys->col_ptr.as<uint32_t>(), N,
+                             maxk == kShortK ? 0u : 32u * kShortK + 1u, (const uint32_t *)rows,
+                             (const uint64_t *)w, lb, sys->row_idx.as<uint32_t>(),
+                             sys->csc_cnt.as<uint32_t>(), sys->csc_wq.as<uint64_t>(), sys->csc_val.as<float>(),
+                             sys->colsum.as<double>(), sys->inv_colsum.as<float>(), flag.as<unsigned int>(),
+                             rhist.as<uint32_t>());
+    };
+    MCS_TRY(wide ? go(segment_merge_kernel<uint64_t, kShortK, W>, 8, kShortK) : go(segment_merge_kernel<uint32_t, kShortK, W>, 4, kShortK));
+    if (longest > 32 * kShortK)
+      MCS_TRY(wide ? go(segment_merge_kernel<uint64_t, 32, W>, 8, 32) : go(segment_merge_kernel<uint32_t, 32, W>, 4, 32));
+  }
+  tmp.release();
+  uint32_t max_count = 0;
+  MCS_CUDA(cudaMemcpyAsync(&max_count, flag.p, sizeof(max_count), cudaMemcpyDeviceToHost, s));
+  // CSR
+  const uint32_t *col_ptr = sys->col_ptr.as<uint32_t>(), *row_idx = sys->row_idx.as<uint32_t>();
+  const uint32_t *csc_cnt = sys->csc_cnt.as<uint32_t>();
+  const uint64_t *csc_wq = sys->csc_wq.as<uint64_t>();
+  MCS_TRY(sys->row_ptr.alloc((size_t)(M + 1) * 4, s));
+  MCS_TRY(exclusive_scan_u32(rhist.as<uint32_t>(), sys->row_ptr.as<uint32_t>(), M + 1, s));
+  MCS_TRY(max_of(rhist, M, flag, &longest, s));  // waits, max_count included
+  if (longest > (uint32_t)kSegLen) return MC_OK;
+  const uint32_t *row_ptr = sys->row_ptr.as<uint32_t>();
+  // the matrix will be finished here: the events are not needed again, and
+  // their buffers hold the entries on their way where they are large enough
+  // (mapping gigabytes of fresh memory costs about 0.7 ms each)
+  const size_t ent_bytes = (size_t)nnz * sizeof(SegEntry<W>);
+  DevBuf ent, part;
+  const auto entry_space = [&](DevBuf &b, DevBuf *old) {
+    if (old && old->bytes >= ent_bytes) { b = std::move(*old); return MC_OK; }
+    return b.alloc(ent_bytes, s);
+  };
+  if (shift > 0) {
+    constexpr int tile = kPartThreads * part_items<W>();
+    const int64_t n_tiles = div_up(nnz, tile);
+    DevBuf starts, tile_col;
+    MCS_TRY(starts.alloc((size_t)kRowBlocks * 4, s));
+    MCS_TRY(tile_col.alloc((size_t)(n_tiles + 1) * 4, s));
+    MCS_TRY(entry_space(part, &key_buf));
+    MCS_TRY(entry_space(ent, weight_buf));
+    count_launch();
+    row_block_starts_kernel<<<1, kRowBlocks, 0, s>>>(row_ptr, M, shift, starts.as<uint32_t>());
+    count_launch();
+    tile_columns_kernel<<<grid_for(n_tiles + 1), 256, 0, s>>>(col_ptr, N, nnz, tile, n_tiles, tile_col.as<uint32_t>());
+    MCS_LAUNCHED();
+    MCS_CUDA(cudaFuncSetAttribute(partition_rows_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(PartSmem<W>)));
+    count_launch();
+    partition_rows_kernel<W><<<(unsigned)n_tiles, kPartThreads, sizeof(PartSmem<W>), s>>>(
+        col_ptr, tile_col.as<uint32_t>(), nnz, row_idx, csc_cnt, csc_wq, shift, starts.as<uint32_t>(),
+        part.as<SegEntry<W>>());
+    MCS_LAUNCHED();
+    constexpr int pad = 80 << 10;
+    MCS_CUDA(cudaFuncSetAttribute(place_rows_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, pad));
+    count_launch();
+    place_rows_kernel<W><<<(unsigned)(((M - 1) >> shift) + 1), kPlaceThreads, pad, s>>>(part.as<SegEntry<W>>(), row_ptr,
+                                                                                      shift, M, ent.as<SegEntry<W>>());
+    MCS_LAUNCHED();
+    part.release();
+  } else {
+    MCS_TRY(entry_space(ent, &key_buf));
+    MCS_CUDA(cudaMemcpyAsync(rhist.p, row_ptr, (size_t)(M + 1) * 4, cudaMemcpyDeviceToDevice, s));
+    MCS_TRY(launch_segments(segment_transpose_kernel<W>, 0, 1, N, s, col_ptr, N, row_idx, csc_cnt, csc_wq,
+                            rhist.as<uint32_t>(), ent.as<SegEntry<W>>()));
+  }
+  key_buf.release();
+  if (W) weight_buf->release();
+  MCS_TRY(sys->col_idx.alloc((size_t)nnz * 4, s));
+  MCS_TRY(sys->csr_cnt.alloc((size_t)nnz * 4, s));
+  MCS_TRY(sys->csr_val.alloc((size_t)nnz * 4, s));
+  if (W) MCS_TRY(sys->csr_wq.alloc((size_t)nnz * 8, s));
+  {
+    const int lb = bits_for(longest - 1);
+    const bool wide = bits_for((uint64_t)N - 1) + lb > 32;
+    auto go = [&](auto *k, size_t kb, int maxk) {
+      return launch_segments(k, kb, maxk, M, s, (const uint32_t *)sys->row_ptr.as<uint32_t>(), M,
+                             maxk == kShortK ? 0u : 32u * kShortK + 1u, (const SegEntry<W> *)ent.as<SegEntry<W>>(), lb, sys->col_idx.as<uint32_t>(),
+                             sys->csr_cnt.as<uint32_t>(), sys->csr_wq.as<uint64_t>(), sys->csr_val.as<float>());
+    };
+    MCS_TRY(wide ? go(segment_rows_kernel<uint64_t, kShortK, W>, 8, kShortK) : go(segment_rows_kernel<uint32_t, kShortK, W>, 4, kShortK));
+    if (longest > 32 * kShortK)
+      MCS_TRY(wide ? go(segment_rows_kernel<uint64_t, 32, W>, 8, 32) : go(segment_rows_kernel<uint32_t, 32, W>, 4, 32));
+  }
+  sys->nnz = nnz;
+  sys->max_count = max_count;
+  sys->values_ready = true;
   *done = true;
   return MC_OK;
 }
@@ -840,7 +1480,7 @@ static int assemble_radix(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t 
   return MC_OK;
 }
 
-int assemble_system(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t s, const uint64_t *weights) {
+int assemble_system(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t s, DevBuf *weights) {
   const uint64_t N = (uint64_t)sys->n_cols;
   // n_v and 1/n_v
   MCS_TRY(sys->n_v.alloc(N * sizeof(uint32_t), s));
@@ -850,15 +1490,22 @@ int assemble_system(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t s, con
   MCS_LAUNCHED();
   sys->weighted = weights != nullptr;
 
-  // 1-4. the CSC and CSR: by buckets where columns and rows are short, else
-  // by a radix sort
-  bool bucketed = false;
-  if (!weights && n > 0 && n < ((int64_t)1 << 31)) MCS_TRY(assemble_buckets(sys, keys.as<uint64_t>(), n, s, &bucketed));
+  // 1-4. the CSC and CSR: by buckets (a thread per column and row) where
+  // columns and rows are short, by sorted segments (a warp each) where they are
+  // longer or weighted, else by a radix sort.  Columns of 16 events and more
+  // on average hardly ever keep below the buckets' 64 everywhere.
+  bool bucketed = false, segmented = false;
+  if (!weights && n > 0 && n < 16 * (int64_t)N && n < ((int64_t)1 << 31))
+    MCS_TRY(assemble_buckets(sys, keys.as<uint64_t>(), n, s, &bucketed));
+  if (!bucketed && n > 0) {
+    MCS_TRY(weights ? assemble_segments<true>(sys, keys, weights, n, s, &segmented)
+                    : assemble_segments<false>(sys, keys, nullptr, n, s, &segmented));
+  }
   if (bucketed) keys.release();
-  else MCS_TRY(assemble_radix(sys, keys, n, s, weights));
+  else if (!segmented) MCS_TRY(assemble_radix(sys, keys, n, s, weights ? weights->as<uint64_t>() : nullptr));
 
   // 5. column sums S_v and the largest count
-  {
+  if (!segmented) {
     MCS_TRY(sys->colsum.alloc(N * sizeof(double), s));
     MCS_TRY(sys->inv_colsum.alloc(N * sizeof(float), s));
     DevBuf mx;
@@ -989,6 +1636,10 @@ template <typename V> static int make_a_values(mc_system *sys, cudaStream_t s) {
 
 int make_values(mc_system *sys, cudaStream_t s) {
   const int64_t nnz = sys->nnz;
+  // assembly by segments has written the float values with the entries
+  const bool ready = sys->values_ready;
+  sys->values_ready = false;
+  if (ready && sys->value_type == MC_VAL_F32) return MC_OK;
   const size_t es = value_storage(sys->value_type) == 0 ? 4 : 2;
   const size_t bytes = (size_t)(nnz > 0 ? nnz : 1) * es;
   MCS_TRY(sys->csr_val.alloc(bytes, s));

@@ -112,6 +112,7 @@ struct mc_system {
   mcs::DevBuf col_ptr, row_idx, csc_cnt;  // u32 [N+1], u32 [nnz], u32 [nnz]
   // projector values (counts as float / half / bfloat16)
   mcs::DevBuf csr_val, csc_val;
+  bool values_ready = false;  // assembly has written the float values
   mcs::DevBuf n_v;      // u32 [N]: histories started in voxel v
   mcs::DevBuf inv_n;    // f32 [N]: 1/n_v (0 if n_v = 0)
   mcs::DevBuf colsum;   // f64 [N]: S_v = sum_j C_jv
@@ -241,9 +242,10 @@ int launch_debug_beam(const TransportSetup &ts, uint64_t n, const double p0[3], 
 
 // Assembly: sorted events -> CSR + CSC + n_v + column sums.  `keys` holds
 // n keys (v*M + j) and is overwritten.
-// `weights` (device, optional): fixed-point weight of each event; the
-// entries are then the weight sums (the system is marked weighted).
-int assemble_system(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t s, const uint64_t *weights = nullptr);
+// `weights` (optional): fixed-point weight of each event; the entries are
+// then the weight sums (the system is marked weighted).  Either buffer may be
+// released.
+int assemble_system(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t s, DevBuf *weights = nullptr);
 
 // Projector value arrays for sys->value_type.
 int make_values(mc_system *sys, cudaStream_t s);
