@@ -171,7 +171,7 @@ static int check_geometry(const mc_geometry *g, const mc_phantom *ph) {
 // the attenuation coefficients, ready for any number of builds.
 struct mc_plan {
   mcs::TransportSetup ts;
-  mcs::DevBuf material, views_d, views_f, coef_d, coef_f, sig_tab, skip;
+  mcs::DevBuf material, views_d, views_f, coef_d, coef_f, sig_tab, cubes;
 };
 
 namespace mcs {
@@ -223,6 +223,12 @@ int build_skip_map(const uint8_t *material, int nx, int ny, int nz, uint8_t *ski
   if (a != skip) MCS_CUDA(cudaMemcpyAsync(skip, a, (size_t)n, cudaMemcpyDeviceToDevice, s));
   MCS_CUDA(cudaStreamSynchronize(s));
   return MC_OK;
+}
+
+// material | distance << 8, for one load per traversal step
+__global__ void pack_cubes_kernel(const uint8_t *mat, const uint8_t *skip, int64_t n, uint16_t *out) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    out[v] = (uint16_t)(mat[v] | (uint32_t)skip[v] << 8);
 }
 
 static int prepare_plan(const mc_phantom *ph, const mc_geometry *g, cudaStream_t s, mc_plan &pl) {
@@ -278,11 +284,18 @@ static int prepare_plan(const mc_phantom *ph, const mc_geometry *g, cudaStream_t
   ts.coef_d_dev = pl.coef_d.as<double>();
   ts.coef_f_dev = pl.coef_f.as<float>();
   ts.sig_tab_dev = pl.sig_tab.as<float>();
-  ts.skip_dev = nullptr;
+  ts.cubes_dev = nullptr;
   if (ts.forced && ts.precision == MC_FP32) {
-    MCS_TRY(pl.skip.alloc(nv, s));
-    MCS_TRY(build_skip_map(ts.material_dev, ts.nx, ts.ny, ts.nz, pl.skip.as<uint8_t>(), s));
-    ts.skip_dev = pl.skip.as<uint8_t>();
+    DevBuf skip;
+    MCS_TRY(skip.alloc(nv, s));
+    MCS_TRY(build_skip_map(ts.material_dev, ts.nx, ts.ny, ts.nz, skip.as<uint8_t>(), s));
+    MCS_TRY(pl.cubes.alloc(nv * sizeof(uint16_t), s));
+    int64_t g = ((int64_t)nv + 255) / 256;
+    if (g > (int64_t)device_sm_count() * 32) g = (int64_t)device_sm_count() * 32;
+    count_launch();
+    pack_cubes_kernel<<<(int)g, 256, 0, s>>>(ts.material_dev, skip.as<uint8_t>(), (int64_t)nv, pl.cubes.as<uint16_t>());
+    MCS_LAUNCHED();
+    ts.cubes_dev = pl.cubes.as<uint16_t>();
   }
   return MC_OK;
 }

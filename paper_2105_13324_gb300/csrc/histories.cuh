@@ -109,16 +109,6 @@ __device__ __forceinline__ Flight fly_once(const TArgs<float> &a, const float2 *
   return f;
 }
 
-// n / d and n mod d by a precomputed floor(2^32 / d) (2^32 - 1 for d = 1): the
-// quotient estimate is the true one or one less.
-__device__ __forceinline__ uint32_t div_magic(uint32_t n, uint32_t d, uint32_t magic, uint32_t &rem) {
-  uint32_t q = __umulhi(n, magic);
-  uint32_t r = n - q * d;
-  if (r >= d) { q += 1u; r -= d; }
-  rem = r;
-  return q;
-}
-
 // Queue an escape that a view may accept (all lanes of the warp call this).
 __device__ __forceinline__ void warp_queue_escape(const TArgs<float> &a, bool want, const Photon &p, uint32_t n_draws,
                                                   int lane) {

@@ -195,7 +195,7 @@ struct TransportSetup {
   const double *coef_d_dev;   // [3*n_mat] 0.1 rho, N_A Z/A, k Z^4 (double)
   const float *coef_f_dev;    // [3*n_mat] 0.1 rho N_A Z/A, 0.1 rho k Z^4, 0 (float)
   const float *sig_tab_dev;   // float path: sigma_KN over the energy window
-  const uint8_t *skip_dev;    // float forced detection: distance map (see build_skip_map), else null
+  const uint16_t *cubes_dev;  // float forced detection: material | distance << 8 (see build_skip_map), else null
   // run
   uint64_t first, count;
   uint32_t key0, key1;

@@ -51,7 +51,7 @@ template <typename T> struct TArgs {
   const T *coef;     // per material: double {0.1 rho, N_A Z/A, k Z^4}; float {0.1 rho N_A Z/A, 0.1 rho k Z^4}
   const T *view_cs;  // [2V] cos, sin of theta_k
   const float *sig_tab;  // [kSigTab] sigma_KN at E_low + i (E0 - E_low)/(kSigTab - 1)
-  const uint8_t *skip;   // float forced detection: distance map of the material grid
+  const uint16_t *cubes;  // float forced detection: material and distance map of the grid
   uint32_t rk[20];   // Philox round keys: round r uses (rk[2r], rk[2r+1])
   int nx, ny, nz, n_mat;
   T h, hx, hy, hz;   // voxel size, half extents
@@ -87,7 +87,7 @@ template <typename T> struct TArgs {
   unsigned long long *work;         // history_kernel: next history not yet taken by a warp
   uint32_t grab;                    // ... histories a warp takes at a time (a multiple of 32)
   uint32_t first_v;                 // ... first mod N
-  uint32_t magic_n, magic_xy, magic_x;  // ... floor(2^32 / d) of N, nx ny, nx (div_magic)
+  uint32_t magic_n, magic_xy, magic_x, magic_views;  // floor(2^32 / d) of N, nx ny, nx, views (div_magic)
 };
 
 // An escaping photon that may pass a collimator: its history, the position
@@ -245,6 +245,16 @@ __device__ __forceinline__ double sigma_kn(double e) {
   const double term2 = l / (2.0 * a);
   const double term3 = (1.0 + 3.0 * a) / (t * t);
   return (2.0 * kPi) * kRe * kRe * (term1 + term2 - term3);
+}
+
+// n / d and n mod d by a precomputed floor(2^32 / d) (2^32 - 1 for d = 1): the
+// quotient estimate is the true one or one less.
+__device__ __forceinline__ uint32_t div_magic(uint32_t n, uint32_t d, uint32_t magic, uint32_t &rem) {
+  uint32_t q = __umulhi(n, magic);
+  uint32_t r = n - q * d;
+  if (r >= d) { q += 1u; r -= d; }
+  rem = r;
+  return q;
 }
 
 // Photon energy with the cross-section quantities that depend on it.
@@ -832,64 +842,6 @@ __device__ __forceinline__ T transmission(const TArgs<T> &a, T px, T py, T pz, T
                                           const T *c0, const T *c1, const T *c2, const float *sig_tab) {
   Energy<T> en;
   en.set(e, a, sig_tab);
-  if constexpr (!is_dbl<T>()) {
-    // float path: the same integral, crossing a whole cube of constant mu per
-    // step.  The distance map gives, for the current voxel, the half-width
-    // D - 1 of the cube around it that holds one material; the ray leaves that
-    // cube at the (D - 1)-th face beyond the voxel's own next face on one
-    // axis, so mu times the length up to there is the exact integral over
-    // the cube (D = 1 is one ordinary voxel step).  Face distances advance by
-    // a constant step per axis, reciprocal multiplies replace divisions, and
-    // the step has no branches.
-    int ix = voxel_index<float>(px, a.hx, a.h, a.inv_h, a.hx_h, a.nx);
-    int iy = voxel_index<float>(py, a.hy, a.h, a.inv_h, a.hy_h, a.ny);
-    int iz = voxel_index<float>(pz, a.hz, a.h, a.inv_h, a.hz_h, a.nz);
-    const int sx = dx > 0.0f ? 1 : (dx < 0.0f ? -1 : 0);
-    const int sy = dy > 0.0f ? 1 : (dy < 0.0f ? -1 : 0);
-    const int sz = dz > 0.0f ? 1 : (dz < 0.0f ? -1 : 0);
-    const float rx = sx ? 1.0f / dx : 0.0f, ry = sy ? 1.0f / dy : 0.0f, rz = sz ? 1.0f / dz : 0.0f;
-    // the first face on an axis lies at (i + (s > 0)) h - half, t = (face - p) / d;
-    // each later face of that axis is h / |d| further along the ray
-    const float ox = -a.hx - px, oy = -a.hy - py, oz = -a.hz - pz;
-    float tx = sx ? fmaf((float)(ix + (sx > 0)), a.h, ox) * rx : INFINITY;
-    float ty = sy ? fmaf((float)(iy + (sy > 0)), a.h, oy) * ry : INFINITY;
-    float tz = sz ? fmaf((float)(iz + (sz > 0)), a.h, oz) * rz : INFINITY;
-    const float dtx = a.h * fabsf(rx), dty = a.h * fabsf(ry), dtz = a.h * fabsf(rz);
-    const float kx_per = fabsf(dx) * a.inv_h, ky_per = fabsf(dy) * a.inv_h, kz_per = fabsf(dz) * a.inv_h;
-    // the ray leaves the grid at the last face of the first axis to run out
-    const float t_grid =
-        fminf(fminf(sx ? fmaf((float)(sx > 0 ? a.nx - 1 - ix : ix), dtx, tx) : INFINITY,
-                    sy ? fmaf((float)(sy > 0 ? a.ny - 1 - iy : iy), dty, ty) : INFINITY),
-              sz ? fmaf((float)(sz > 0 ? a.nz - 1 - iz : iz), dtz, tz) : INFINITY);
-    const int nx = a.nx, ny = a.ny;
-    int lin = (iz * ny + iy) * nx + ix;
-    float t = 0.0f, sum = 0.0f;
-    const int max_steps = a.nx + a.ny + a.nz + 3;
-    for (int it = 0; it < max_steps; ++it) {
-      const int m = __ldg(a.mat + lin);
-      const int D = __ldg(a.skip + lin);
-      const float e = (float)(D - 1);
-      const float cx = fmaf(e, dtx, tx), cy = fmaf(e, dty, ty), cz = fmaf(e, dtz, tz);
-      const float tc = fminf(fminf(fminf(cx, cy), cz), t_grid);
-      sum = fmaf(mu_total<float>(c0, c1, c2, m, en), fmaxf(tc - t, 0.0f), sum);
-      t = fmaxf(t, tc);
-      if (tc >= t_grid) break;
-      // faces crossed on each axis up to tc: all D on the axis that leaves
-      // the cube, floor((tc - t_axis) / step) + 1 on the others
-      const int kx = cx == tc ? D : (tx <= tc ? min((int)((tc - tx) * kx_per) + 1, D) : 0);
-      const int ky = cy == tc ? D : (ty <= tc ? min((int)((tc - ty) * ky_per) + 1, D) : 0);
-      const int kz = cz == tc ? D : (tz <= tc ? min((int)((tc - tz) * kz_per) + 1, D) : 0);
-      ix += sx * kx;
-      iy += sy * ky;
-      iz += sz * kz;
-      if ((unsigned)ix >= (unsigned)a.nx || (unsigned)iy >= (unsigned)a.ny || (unsigned)iz >= (unsigned)a.nz) break;
-      tx = fmaf((float)kx, dtx, tx);
-      ty = fmaf((float)ky, dty, ty);
-      tz = fmaf((float)kz, dtz, tz);
-      lin = (iz * ny + iy) * nx + ix;
-    }
-    return __expf(-sum);
-  }
   int ix = voxel_index<T>(px, a.hx, a.h, a.inv_h, a.hx_h, a.nx);
   int iy = voxel_index<T>(py, a.hy, a.h, a.inv_h, a.hy_h, a.ny);
   int iz = voxel_index<T>(pz, a.hz, a.h, a.inv_h, a.hz_h, a.nz);
@@ -929,8 +881,7 @@ __device__ __forceinline__ T transmission(const TArgs<T> &a, T px, T py, T pz, T
       tz = face(iz, sz, a.hz, pz, dz);
     }
   }
-  if constexpr (is_dbl<T>()) return exp(-sum);
-  else return __expf(-sum);
+  return exp(-sum);
 }
 
 // Klein-Nishina angular density of the scattered direction per steradian,
@@ -955,7 +906,8 @@ template <typename T> __device__ __forceinline__ T kn_pdf_sr(T e, T mu, const En
 // copy's own Philox block (counter (k, 1 + n, h_lo, h_hi)), weighted by
 // the survival at the interaction, the angular probability of that
 // direction, the collimator's open fraction and the transmission to the
-// grid boundary, then binned like an analog detection.
+// grid boundary, then binned like an analog detection.  The double path's;
+// forced.cuh has the float one.
 template <typename T>
 __device__ __forceinline__ void fd_copy(const TArgs<T> &a, const FdRec<T> &r, int k, const T *c0, const T *c1,
                                         const T *c2, const float *sig_tab) {
@@ -964,16 +916,8 @@ __device__ __forceinline__ void fd_copy(const TArgs<T> &a, const FdRec<T> &r, in
   const T u0 = uniform<T>(w0), u1 = uniform<T>(w1), u2 = uniform<T>(w2), u3 = uniform<T>(w3);
   const T ck = a.view_cs[2 * k], sk = a.view_cs[2 * k + 1];
   T ct, st;
-  if constexpr (is_dbl<T>()) {
-    ct = 1.0 - u0 * (1.0 - a.cos_max);
-    st = sqrt0<double>(1.0 - ct * ct);
-  } else {
-    // 1 - cos is a few 1e-3 at most: sin^2 = (1 - cos)(1 + cos) keeps float's
-    // relative precision where 1 - cos^2 would cancel
-    const float om = u0 * a.one_m_cos_max;
-    ct = 1.0f - om;
-    st = sqrt0<float>(om * (2.0f - om));
-  }
+  ct = 1.0 - u0 * (1.0 - a.cos_max);
+  st = sqrt0<double>(1.0 - ct * ct);
   T cph, sph;
   cos_sin_2pi<T>(u1, cph, sph);
   const T dx = ct * ck - st * cph * sk, dy = ct * sk + st * cph * ck, dz = st * sph;
@@ -986,12 +930,8 @@ __device__ __forceinline__ void fd_copy(const TArgs<T> &a, const FdRec<T> &r, in
     e1 = r.e;
   } else {
     const T mu_s = r.d[0] * dx + r.d[1] * dy + r.d[2] * dz;
-    if constexpr (is_dbl<T>()) {
-      const double eps = 1.0 / (1.0 + (r.e / kMec2) * (1.0 - mu_s));
-      e1 = eps * r.e;
-    } else {
-      e1 = __fdividef(r.e, 1.0f + r.e * (float)(1.0 / kMec2) * (1.0f - mu_s));
-    }
+    const double eps = 1.0 / (1.0 + (r.e / kMec2) * (1.0 - mu_s));
+    e1 = eps * r.e;
     if (e1 < a.e_low) return;
     Energy<T> en;
     en.set(r.e, a, sig_tab);
@@ -1005,8 +945,7 @@ __device__ __forceinline__ void fd_copy(const TArgs<T> &a, const FdRec<T> &r, in
   T au = -qx * sk + qy * ck;
   T bv = qz;
   T rr;
-  if constexpr (is_dbl<T>()) rr = sqrt(-2.0 * log(u2));
-  else rr = sqrt0<float>(-2.0f * __logf(u2));
+  rr = sqrt(-2.0 * log(u2));
   T cb, sb;
   cos_sin_2pi<T>(u3, cb, sb);
   au += a.sigma * (rr * cb);
@@ -1178,7 +1117,7 @@ template <typename T> void make_targs(const TransportSetup &ts, TArgs<T> &a) {
   a.view_cs = std::is_same<T, double>::value ? (const T *)(const void *)ts.view_cs_dev
                                              : (const T *)(const void *)ts.view_cs_f_dev;
   a.sig_tab = ts.sig_tab_dev;
-  a.skip = ts.skip_dev;
+  a.cubes = ts.cubes_dev;
   round_keys(ts.key0, ts.key1, a.rk);
   a.nx = ts.nx; a.ny = ts.ny; a.nz = ts.nz; a.n_mat = ts.n_mat;
   a.h = (T)ts.h;
@@ -1234,6 +1173,7 @@ template <typename T> void make_targs(const TransportSetup &ts, TArgs<T> &a) {
   a.magic_n = magic(a.n_vox);
   a.magic_xy = magic((uint32_t)ts.nx * (uint32_t)ts.ny);
   a.magic_x = magic((uint32_t)ts.nx);
+  a.magic_views = magic((uint32_t)ts.n_views);
   const double cos_max = 1.0 / std::sqrt(1.0 + tan_max * tan_max);
   const double omega = 2.0 * kPi * (1.0 - cos_max);
   a.cos_max = (T)cos_max;
@@ -1246,14 +1186,12 @@ template <typename T> void make_targs(const TransportSetup &ts, TArgs<T> &a) {
   a.q_dir = (unsigned long long)std::llrint(band * kFdScale);
 }
 
+int launch_rays(const TransportSetup &ts, TArgs<float> &a, cudaStream_t s);  // forced.cuh
+
 template <typename T> int launch_transport_t(const TransportSetup &ts, cudaStream_t s) {
   TArgs<T> a;
   make_targs<T>(ts, a);
   if (ts.count == 0) return MC_OK;
-  if (ts.forced && !is_dbl<T>() && !ts.skip_dev) {
-    set_error("float forced detection needs the plan's distance map");
-    return MC_EINVAL;
-  }
   const int threads = 256;
   int per_sm = 0;
   if (ts.forced) {
@@ -1280,7 +1218,10 @@ template <typename T> int launch_transport_t(const TransportSetup &ts, cudaStrea
   MCS_LAUNCHED();
   if (ts.ev_mid) MCS_CUDA(cudaEventRecord(ts.ev_mid, s));
   const int dgrid = device_sm_count() * 8;
-  if (ts.forced) { count_launch(); fd_kernel<T><<<dgrid, 256, 0, s>>>(a); }
+  if (ts.forced) {
+    if constexpr (is_dbl<T>()) { count_launch(); fd_kernel<T><<<dgrid, 256, 0, s>>>(a); }
+    else return launch_rays(ts, a, s);
+  }
   else if (ts.records) { count_launch(); detect_kernel<T, true><<<dgrid, 256, 0, s>>>(a); }
   else if constexpr (is_dbl<T>()) { count_launch(); detect_kernel<T, false><<<dgrid, 256, 0, s>>>(a); }
   MCS_LAUNCHED();

@@ -1,6 +1,8 @@
 // transport_f32.cu -- production (float) transport: the analog photon-history
-// kernel of histories.cuh, and transport.cuh's float instantiations (forced
-// detection, per-history traces).
+// kernel of histories.cuh, the forced-detection rays of forced.cuh, and
+// transport.cuh's float instantiations (the interaction queue, per-history
+// traces).
+#include "forced.cuh"
 #include "histories.cuh"
 
 namespace mcs {
