@@ -286,7 +286,7 @@ MC_API int mc_system_set_value_type(mc_system *sys, int32_t value_type, int32_t 
  * (back-projection, CSC) each 0 = streaming layout (entries of runs of whole
  * rows staged in shared memory, then one fixed-order sum per row: warps of
  * 32 R rows, R = 1, 2 or 4 rows per lane, when rows average fewer than 16
- * entries, else one warp per row in tiles of ~4096 entries), 1, 2, 4, 8,
+ * entries, else a thread per row in tiles of ~4096 entries), 1, 2, 4, 8,
  * 16 or 32 = that many lanes per row (column), or -1 = keep.  Every layout
  * gives the same sums up to FP32 rounding order.  The streaming layout needs
  * every row (column) shorter than 2048 entries: MC_EINVAL otherwise (the
@@ -405,7 +405,7 @@ MC_API int mc_system_autotune(mc_system *sys, void *stream);
  * captured once into a CUDA graph per n_iter and replayed.  Every system
  * must be a full (not ordered-subset) FP32 system, of any projector layout:
  * the batch makes its own work units over each system's non-empty rows and
- * columns (warp chunks; tiles of one warp per row where rows or columns
+ * columns (warp chunks; tiles of whole rows where rows or columns
  * average 16 or more entries, which then must be shorter than 2048 entries,
  * else MC_EINVAL).  Results equal mlem_iterate's up to FP32 rounding order.
  * Systems in a batch must not be used by other calls while it runs. */

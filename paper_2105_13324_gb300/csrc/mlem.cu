@@ -326,10 +326,9 @@ __global__ void sensitivity_kernel(const double *colsum, const uint32_t *n_v, in
 // CSR (CSC) arrays.  The block first reads the tile's entries and gathers the
 // vector with independent, coalesced loads (many requests in flight), keeps
 // the products in shared memory, and then reduces each row from shared
-// memory: one warp per row (segments of 16 or more entries on average), or
-// one thread per row (the batch kernels).  Single systems with shorter
-// segments use the warp chunks below instead.  Every row is summed in a fixed
-// order, so results are reproducible.
+// memory, a thread per row.  Segments of fewer than 16 entries on average use
+// the warp chunks below instead.  Every row is summed in a fixed order, so
+// results are reproducible.
 constexpr int kStreamTile = 4096;
 constexpr int kStreamThreads = 256;
 
@@ -365,63 +364,58 @@ __device__ __forceinline__ void stream_products(uint32_t p0, uint32_t cnt, const
   }
 }
 
-// Sum of the products of segment [b, e) of the tile: one thread, or the 32
-// lanes of a warp (result in every lane).
-template <bool WARP>
-__device__ __forceinline__ float stream_segment(const float *s_prod, uint32_t b, uint32_t e) {
-  float acc = 0.0f;
-  if (WARP) {
-    for (uint32_t k = b + (threadIdx.x & 31); k < e; k += 32) acc += s_prod[k];
+// Sum of the products [b, e) of a segment by one thread, as 32 partial sums
+// with stride 32 and then the butterfly over them (offsets 16, 8, 4, 2, 1): the
+// order of a warp whose lanes take every 32nd product, without its 31 idle
+// lanes.
+__device__ __forceinline__ float strided_tree(const float *s_prod, uint32_t b, uint32_t e) {
+  float a[16];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  } else {
-    for (uint32_t k = b; k < e; ++k) acc += s_prod[k];
+  for (uint32_t i = 0; i < 16; ++i) {
+    float u = 0.0f, w = 0.0f;
+    for (uint32_t k = b + i; k < e; k += 32) {
+      u += s_prod[k];
+      if (k + 16 < e) w += s_prod[k + 16];
+    }
+    a[i] = u + w;
   }
-  return acc;
+#pragma unroll
+  for (uint32_t o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (uint32_t i = 0; i < o; ++i) a[i] += a[i + o];
+  return a[0];
 }
 
-// Reduces every segment j in [j0, j1) of the tile from shared memory and
-// hands its sum to out.store(j, acc, out.load(j), segment j non-empty).  Warp
-// mode: one warp per
-// segment.  Thread mode: each thread takes kSegBatch segments kStreamThreads
-// apart and issues their pointer loads and out.load() before any reduction,
-// so that short segments do not leave one load in flight per thread.
-constexpr int kSegBatch = 4;
+// Reduces every segment j in [j0, j1) of the tile from shared memory, a thread
+// each, and hands its sum to out.store(j, acc, out.load(j), segment j
+// non-empty).  (A warp per segment, the former reduction, was a chain of five
+// shuffles and a dependent pointer load per segment for 17 to 26 segments one
+// after another: at rows of 18 entries on the 128^3 system 0.262 ms a forward
+// projection against 0.168; at 31, 0.336
+// against 0.267.)
 template <typename Out>
-__device__ __forceinline__ void stream_segments_thread(const uint32_t *__restrict__ ptr, uint32_t j0, uint32_t j1,
-                                                       uint32_t p0, const float *s_prod, Out &out) {
-  for (uint32_t base = j0 + threadIdx.x; base < j1; base += kSegBatch * kStreamThreads) {
-    uint32_t b[kSegBatch], e[kSegBatch];
-    typename Out::Pre pre[kSegBatch] = {};
-#pragma unroll
-    for (int u = 0; u < kSegBatch; ++u) {
-      const uint32_t j = base + u * kStreamThreads;
-      b[u] = e[u] = p0;
-      if (j < j1) {
-        b[u] = ptr[j];
-        e[u] = ptr[j + 1];
-        pre[u] = out.load(j);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kSegBatch; ++u) {
-      const uint32_t j = base + u * kStreamThreads;
-      if (j < j1) out.store(j, stream_segment<false>(s_prod, b[u] - p0, e[u] - p0), pre[u], e[u] > b[u]);
-    }
-  }
-}
-
-template <bool WARP, typename Out>
 __device__ __forceinline__ void stream_segments(const uint32_t *__restrict__ ptr, uint32_t j0, uint32_t j1,
                                                 uint32_t p0, const float *s_prod, Out &out) {
-  if (WARP) {
-    for (uint32_t j = j0 + (threadIdx.x >> 5); j < j1; j += kStreamThreads / 32) {
-      const uint32_t b = ptr[j], e = ptr[j + 1];
-      const float acc = stream_segment<true>(s_prod, b - p0, e - p0);
-      if ((threadIdx.x & 31) == 0) out.store(j, acc, out.load(j), e > b);
-    }
-  } else {
-    stream_segments_thread(ptr, j0, j1, p0, s_prod, out);
+  for (uint32_t j = j0 + threadIdx.x; j < j1; j += kStreamThreads) {
+    const uint32_t b = ptr[j], e = ptr[j + 1];
+    const typename Out::Pre pre = out.load(j);
+    out.store(j, strided_tree(s_prod, b - p0, e - p0), pre, e > b);
+  }
+}
+
+// The same sums by a warp per segment: the batch kernels keep it, whose other
+// path (warp chunks, all serving systems take it) would lose a tenth to the
+// registers of the 16 partial sums.
+template <typename Out>
+__device__ __forceinline__ void stream_segments_warp(const uint32_t *__restrict__ ptr, uint32_t j0, uint32_t j1,
+                                                     uint32_t p0, const float *s_prod, Out &out) {
+  for (uint32_t j = j0 + (threadIdx.x >> 5); j < j1; j += kStreamThreads / 32) {
+    const uint32_t b = ptr[j], e = ptr[j + 1];
+    float acc = 0.0f;
+    for (uint32_t k = b - p0 + (threadIdx.x & 31); k < e - p0; k += 32) acc += s_prod[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) out.store(j, acc, out.load(j), e > b);
   }
 }
 
@@ -478,7 +472,7 @@ struct BackOut {
   }
 };
 
-template <typename V, bool WARP, int MODE, bool LL>
+template <typename V, int MODE, bool LL>
 __global__ void __launch_bounds__(kStreamThreads) stream_forward_kernel(const uint32_t *__restrict__ row_ptr,
                                                                      const uint32_t *__restrict__ tiles,
                                                                      const uint32_t *__restrict__ col,
@@ -490,19 +484,20 @@ __global__ void __launch_bounds__(kStreamThreads) stream_forward_kernel(const ui
                                                                      const float *__restrict__ add) {
   __shared__ float s_prod[kStreamTile];
   __shared__ double s_tmp[kStreamThreads / 32];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t r0 = tiles[blockIdx.x], r1 = tiles[blockIdx.x + 1];
   const uint32_t p0 = row_ptr[r0];
   stream_products<V>(p0, row_ptr[r1] - p0, col, val, xs, s_prod);
   __syncthreads();
   FwdOut<MODE, LL> o{y, out, rmap, add, 0.0};
-  stream_segments<WARP>(row_ptr, r0, r1, p0, s_prod, o);
+  stream_segments(row_ptr, r0, r1, p0, s_prod, o);
   if (LL) {
     const double t = block_sum_double(o.ll, s_tmp);
     if (threadIdx.x == 0) partials[blockIdx.x] = t;
   }
 }
 
-template <typename V, bool WARP, int MODE>
+template <typename V, int MODE>
 __global__ void __launch_bounds__(kStreamThreads) stream_back_kernel(const uint32_t *__restrict__ col_ptr,
                                                                   const uint32_t *__restrict__ tiles,
                                                                   const uint32_t *__restrict__ row,
@@ -512,12 +507,13 @@ __global__ void __launch_bounds__(kStreamThreads) stream_back_kernel(const uint3
                                                                   const float *__restrict__ inv_colsum,
                                                                   float *__restrict__ x, float *__restrict__ xs) {
   __shared__ float s_prod[kStreamTile];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t c0 = tiles[blockIdx.x], c1 = tiles[blockIdx.x + 1];
   const uint32_t p0 = col_ptr[c0];
   stream_products<V>(p0, col_ptr[c1] - p0, row, val, r, s_prod);
   __syncthreads();
   BackOut<MODE> o{inv_n, inv_colsum, x, xs};
-  stream_segments<WARP>(col_ptr, c0, c1, p0, s_prod, o);
+  stream_segments(col_ptr, c0, c1, p0, s_prod, o);
 }
 
 // ---------------------------------------------------------------------------
@@ -756,8 +752,7 @@ static void stream_fwd_launch(const mc_system *sys, const float *xs, const float
   const V *val = sys->csr_val.as<V>();
   count_launch();
   if (sys->warp_rows_fwd)
-    stream_forward_kernel<V, true, MODE, LL><<<nb, kStreamThreads, 0, s>>>(rp, t, ci, val, xs, y, out, partials,
-                                                                            rmap, add);
+    launch_pdl(stream_forward_kernel<V, MODE, LL>, nb, kStreamThreads, s, rp, t, ci, val, xs, y, out, partials, rmap, add);
   else {
     const int R = chunk_rows_per_lane(sys->nnz, sys->n_rows, sys->n_rows);
     const unsigned g = (unsigned)div_up(sys->n_rows, (int64_t)kChunkThreads * R);
@@ -777,7 +772,7 @@ static void stream_back_launch(const mc_system *sys, const float *r, float *x, f
   const float *inv_n = scale ? scale : proj_scale(sys), *ics = proj_inv_norm(sys);
   count_launch();
   if (sys->warp_rows_bwd)
-    stream_back_kernel<V, true, MODE><<<nb, kStreamThreads, 0, s>>>(cp, t, ri, val, r, inv_n, ics, x, xs);
+    launch_pdl(stream_back_kernel<V, MODE>, nb, kStreamThreads, s, cp, t, ri, val, r, inv_n, ics, x, xs);
   else {
     const int R = chunk_rows_per_lane(sys->nnz, sys->n_cols, sys->n_cols);
     const unsigned g = (unsigned)div_up(sys->n_cols, (int64_t)kChunkThreads * R);
@@ -1314,9 +1309,8 @@ int pgd_step(int64_t n, double alpha, const double *sens, const float *bp, const
 // of all systems and one back-projection launch over their CSC units; a
 // block finds its system by binary search in the prefix of unit counts.  A
 // unit is 256 R consecutive rows (columns) as eight warp chunks, or, for a
-// system whose rows (columns) average 16 or more entries, one tile with a
-// warp per row (column).  The
-// whole reconstruction (start images, n_iter iterations, write-back of the
+// system whose rows (columns) average 16 or more entries, one tile of whole
+// rows (columns).  The whole reconstruction (start images, n_iter iterations, write-back of the
 // images) is captured once in a CUDA graph and replayed.
 //
 // Serving systems are built from few histories, so most of their rows and
@@ -1344,7 +1338,7 @@ struct BatchSys {
   float *x_c, *xs_c;         // per non-empty column: image, image / n_v
   const float *ics_c, *invn_c;  // per non-empty column: 1 / S_v, 1 / n_v
   int64_t n_rows, n_cols, m_c, n_c;
-  int warp_fwd, warp_bwd;  // tiles with a warp per segment, else warp chunks
+  int warp_fwd, warp_bwd;  // tiles of whole segments, else warp chunks
   int rpl_fwd, rpl_bwd;    // warp chunks: segments per lane
 };
 
@@ -1410,7 +1404,7 @@ __device__ __forceinline__ void batch_forward_tile(const BatchSys *__restrict__ 
   const uint32_t p0 = ptr[j0];
   stream_products<float>(p0, ptr[j1] - p0, S.col_idx, S.csr_val, S.xs_c, s_prod);
   __syncthreads();
-  stream_segments<true>(ptr, j0, j1, p0, s_prod, o);
+  stream_segments_warp(ptr, j0, j1, p0, s_prod, o);
 }
 
 __device__ __forceinline__ void batch_back_tile(const BatchSys *__restrict__ systems,
@@ -1428,7 +1422,7 @@ __device__ __forceinline__ void batch_back_tile(const BatchSys *__restrict__ sys
   const uint32_t p0 = ptr[j0];
   stream_products<float>(p0, ptr[j1] - p0, S.row_idx, S.csc_val, S.r_c, s_prod);
   __syncthreads();
-  stream_segments<true>(ptr, j0, j1, p0, s_prod, o);
+  stream_segments_warp(ptr, j0, j1, p0, s_prod, o);
 }
 
 __global__ void __launch_bounds__(kStreamThreads) batch_forward_kernel(const BatchSys *__restrict__ systems,
