@@ -329,6 +329,17 @@ template <> __device__ __forceinline__ float uniform<float>(uint32_t w) {
   return (__uint_as_float(0x3F800000u | (w >> 9)) - 1.0f) + 5.9604644775390625e-8f;
 }
 
+// n / d and n mod d by a precomputed floor(2^32 / d) (2^32 - 1 for d = 1): the
+// quotient estimate is the true one or one less.
+__device__ __forceinline__ uint32_t div_magic(uint32_t n, uint32_t d, uint32_t magic, uint32_t &rem) {
+  uint32_t q = __umulhi(n, magic);
+  uint32_t r = n - q * d;
+  if (r >= d) { q += 1u; r -= d; }
+  rem = r;
+  return q;
+}
+inline uint32_t div_magic_of(uint32_t d) { return d <= 1u ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d); }
+
 inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 int device_sm_count();

@@ -247,16 +247,6 @@ __device__ __forceinline__ double sigma_kn(double e) {
   return (2.0 * kPi) * kRe * kRe * (term1 + term2 - term3);
 }
 
-// n / d and n mod d by a precomputed floor(2^32 / d) (2^32 - 1 for d = 1): the
-// quotient estimate is the true one or one less.
-__device__ __forceinline__ uint32_t div_magic(uint32_t n, uint32_t d, uint32_t magic, uint32_t &rem) {
-  uint32_t q = __umulhi(n, magic);
-  uint32_t r = n - q * d;
-  if (r >= d) { q += 1u; r -= d; }
-  rem = r;
-  return q;
-}
-
 // Photon energy with the cross-section quantities that depend on it.
 template <typename T> struct Energy {
   T e, sig, e3, ie3;
@@ -1169,11 +1159,10 @@ template <typename T> void make_targs(const TransportSetup &ts, TArgs<T> &a) {
   a.weights = ts.weights;
   a.work = ts.work;
   a.first_v = (uint32_t)(ts.first % a.n_vox);
-  const auto magic = [](uint32_t d) { return d <= 1u ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d); };
-  a.magic_n = magic(a.n_vox);
-  a.magic_xy = magic((uint32_t)ts.nx * (uint32_t)ts.ny);
-  a.magic_x = magic((uint32_t)ts.nx);
-  a.magic_views = magic((uint32_t)ts.n_views);
+  a.magic_n = div_magic_of(a.n_vox);
+  a.magic_xy = div_magic_of((uint32_t)ts.nx * (uint32_t)ts.ny);
+  a.magic_x = div_magic_of((uint32_t)ts.nx);
+  a.magic_views = div_magic_of((uint32_t)ts.n_views);
   const double cos_max = 1.0 / std::sqrt(1.0 + tan_max * tan_max);
   const double omega = 2.0 * kPi * (1.0 - cos_max);
   a.cos_max = (T)cos_max;
