@@ -536,7 +536,13 @@ __global__ void __launch_bounds__(kStreamThreads) stream_back_kernel(const uint3
 // block.
 constexpr int kChunkWindow = 128;
 constexpr int kChunkThreads = 128;
-static_assert(kStreamTile >= (kStreamThreads / 32) * kChunkWindow, "a tile block's products hold its warps' windows");
+// The batch kernels' window: with four rows a lane (rows of 1.1 entries) a
+// chunk holds ~140 entries, one window of 160 where 128 takes two, the second
+// nearly empty: 64 mixed systems, 30 iterations, 3.47 -> 3.22 ms (192 entries
+// 3.51, 256 3.59: registers), and 3.16 with the smaller shared memory of
+// batches without tiles.
+constexpr int kBatchWindow = 160;
+static_assert(kStreamTile >= (kStreamThreads / 32) * kBatchWindow, "a tile block's products hold its warps' windows");
 
 // Segments per lane for n segments averaging nnz / n entries, in a launch
 // over `launch_segments` segments in all.
@@ -549,7 +555,7 @@ inline int chunk_rows_per_lane(int64_t nnz, int64_t n, int64_t launch_segments) 
 
 // j0: the warp's first segment (a multiple of 32 R); s_w: the warp's
 // kChunkWindow floats.
-template <int R, typename V, typename Out>
+template <int R, typename V, int W = kChunkWindow, typename Out>
 __device__ __forceinline__ void chunk_segments(const uint32_t *__restrict__ ptr, int64_t n_seg,
                                                const uint32_t *__restrict__ idx, const V *__restrict__ val,
                                                const float *__restrict__ vec, float *s_w, Out &out, int64_t j0) {
@@ -569,14 +575,14 @@ __device__ __forceinline__ void chunk_segments(const uint32_t *__restrict__ ptr,
   }
   // the chunk's entries [p0, p1): lane 0's first to lane 31's last
   const uint32_t p0 = __shfl_sync(0xffffffffu, b[0], 0), p1 = __shfl_sync(0xffffffffu, e[R - 1], 31);
-  for (uint32_t w0 = p0; w0 < p1; w0 += kChunkWindow) {
-    const uint32_t n = min((uint32_t)kChunkWindow, p1 - w0);
+  for (uint32_t w0 = p0; w0 < p1; w0 += W) {
+    const uint32_t n = min((uint32_t)W, p1 - w0);
     const uint32_t *ip = idx + w0 + lane;
     const V *vp = val + w0 + lane;
-    uint32_t c[kChunkWindow / 32];
-    float v[kChunkWindow / 32];
+    uint32_t c[W / 32];
+    float v[W / 32];
 #pragma unroll
-    for (int u = 0; u < kChunkWindow / 32; ++u) {
+    for (int u = 0; u < W / 32; ++u) {
       c[u] = 0u;
       v[u] = 0.0f;
       if (lane + 32u * u < n) {
@@ -585,7 +591,7 @@ __device__ __forceinline__ void chunk_segments(const uint32_t *__restrict__ ptr,
       }
     }
 #pragma unroll
-    for (int u = 0; u < kChunkWindow / 32; ++u)
+    for (int u = 0; u < W / 32; ++u)
       if (lane + 32u * u < n) s_w[lane + 32 * u] = v[u] * __ldg(vec + c[u]);
     __syncwarp();
 #pragma unroll
@@ -1524,15 +1530,16 @@ __device__ __forceinline__ void batch_chunks(const uint32_t *__restrict__ ptr, i
                                              const uint32_t *__restrict__ idx, const float *__restrict__ val,
                                              const float *__restrict__ vec, float *s_prod, Out &o, uint32_t u,
                                              int R) {
-  float *s_w = s_prod + (threadIdx.x >> 5) * kChunkWindow;
+  float *s_w = s_prod + (threadIdx.x >> 5) * kBatchWindow;
   const int64_t j0 = ((int64_t)u * kStreamThreads + (threadIdx.x & ~31u)) * R;
-  if (R == 1) chunk_segments<1, float>(ptr, n_seg, idx, val, vec, s_w, o, j0);
-  else if (R == 2) chunk_segments<2, float>(ptr, n_seg, idx, val, vec, s_w, o, j0);
-  else chunk_segments<4, float>(ptr, n_seg, idx, val, vec, s_w, o, j0);
+  if (R == 1) chunk_segments<1, float, kBatchWindow>(ptr, n_seg, idx, val, vec, s_w, o, j0);
+  else if (R == 2) chunk_segments<2, float, kBatchWindow>(ptr, n_seg, idx, val, vec, s_w, o, j0);
+  else chunk_segments<4, float, kBatchWindow>(ptr, n_seg, idx, val, vec, s_w, o, j0);
 }
 
 // One forward (ratio) tile and one back-projection (EM update) tile of the
 // batch, by global tile index t
+template <bool TILES>
 __device__ __forceinline__ void batch_forward_tile(const BatchSys *__restrict__ systems,
                                                    const uint64_t *__restrict__ tile_off, int n_sys, uint64_t t,
                                                    float *s_prod, BatchSys *s_desc) {
@@ -1540,7 +1547,7 @@ __device__ __forceinline__ void batch_forward_tile(const BatchSys *__restrict__ 
   const BatchSys &S = batch_desc(systems, tile_off, n_sys, s_desc, t, tile);
   const uint32_t *__restrict__ ptr = S.row_ptr;
   BatchFwdOut o{S.y_c, S.r_c};
-  if (!S.warp_fwd) {  // warp chunks over rows [256 R u, 256 R (u + 1))
+  if (!TILES || !S.warp_fwd) {  // warp chunks over rows [256 R u, 256 R (u + 1))
     batch_chunks(ptr, S.m_c, S.col_idx, S.csr_val, S.xs_c, s_prod, o, tile, S.rpl_fwd);
     return;
   }
@@ -1551,6 +1558,7 @@ __device__ __forceinline__ void batch_forward_tile(const BatchSys *__restrict__ 
   stream_segments_warp(ptr, j0, j1, p0, s_prod, o);
 }
 
+template <bool TILES>
 __device__ __forceinline__ void batch_back_tile(const BatchSys *__restrict__ systems,
                                                 const uint64_t *__restrict__ tile_off, int n_sys, uint64_t t,
                                                 float *s_prod, BatchSys *s_desc) {
@@ -1558,7 +1566,7 @@ __device__ __forceinline__ void batch_back_tile(const BatchSys *__restrict__ sys
   const BatchSys &S = batch_desc(systems, tile_off, n_sys, s_desc, t, tile);
   const uint32_t *__restrict__ ptr = S.col_ptr;
   BackOut<1> o{S.invn_c, S.ics_c, S.x_c, S.xs_c};
-  if (!S.warp_bwd) {  // warp chunks over columns [256 R u, 256 R (u + 1))
+  if (!TILES || !S.warp_bwd) {  // warp chunks over columns [256 R u, 256 R (u + 1))
     batch_chunks(ptr, S.n_c, S.row_idx, S.csc_val, S.r_c, s_prod, o, tile, S.rpl_bwd);
     return;
   }
@@ -1569,21 +1577,27 @@ __device__ __forceinline__ void batch_back_tile(const BatchSys *__restrict__ sys
   stream_segments_warp(ptr, j0, j1, p0, s_prod, o);
 }
 
+// TILES: some system of the batch has tiles.  Without (no serving system has),
+// the kernels need neither a tile's shared memory nor its registers.
+template <bool TILES> constexpr int batch_floats() { return TILES ? kStreamTile : (kStreamThreads / 32) * kBatchWindow; }
+
+template <bool TILES>
 __global__ void __launch_bounds__(kStreamThreads) batch_forward_kernel(const BatchSys *__restrict__ systems,
                                                                     const uint64_t *__restrict__ tile_off,
                                                                     int n_sys) {
-  __shared__ float s_prod[kStreamTile];
+  __shared__ float s_prod[batch_floats<TILES>()];
   __shared__ BatchSys s_desc;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  batch_forward_tile(systems, tile_off, n_sys, blockIdx.x, s_prod, &s_desc);
+  batch_forward_tile<TILES>(systems, tile_off, n_sys, blockIdx.x, s_prod, &s_desc);
 }
 
+template <bool TILES>
 __global__ void __launch_bounds__(kStreamThreads) batch_back_kernel(const BatchSys *__restrict__ systems,
                                                                  const uint64_t *__restrict__ tile_off, int n_sys) {
-  __shared__ float s_prod[kStreamTile];
+  __shared__ float s_prod[batch_floats<TILES>()];
   __shared__ BatchSys s_desc;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  batch_back_tile(systems, tile_off, n_sys, blockIdx.x, s_prod, &s_desc);
+  batch_back_tile<TILES>(systems, tile_off, n_sys, blockIdx.x, s_prod, &s_desc);
 }
 
 // All n_iter iterations of every system in one cooperative launch: the
@@ -1601,12 +1615,12 @@ __global__ void __launch_bounds__(kStreamThreads) batch_persistent_kernel(const 
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   for (int it = 0; it < n_iter; ++it) {
     for (uint64_t t = blockIdx.x; t < n_fwd; t += gridDim.x) {
-      batch_forward_tile(systems, tile_fwd, n_sys, t, s_prod, &s_desc);
+      batch_forward_tile<true>(systems, tile_fwd, n_sys, t, s_prod, &s_desc);
       __syncthreads();  // s_prod and s_desc are reused by the next tile
     }
     grid.sync();
     for (uint64_t t = blockIdx.x; t < n_bwd; t += gridDim.x) {
-      batch_back_tile(systems, tile_bwd, n_sys, t, s_prod, &s_desc);
+      batch_back_tile<true>(systems, tile_bwd, n_sys, t, s_prod, &s_desc);
       __syncthreads();
     }
     grid.sync();
@@ -1729,6 +1743,7 @@ struct mc_batch {
   mcs::DevBuf systems, tile_fwd, tile_bwd, x0, part_y, part_s;
   std::vector<mcs::DevBuf> owned;  // kBatchBufs per system
   uint64_t n_tiles_fwd = 0, n_tiles_bwd = 0;
+  bool tiles_fwd = false, tiles_bwd = false;  // some system has tiles (else all are warp chunks)
   cudaGraphExec_t exec = nullptr;
   int exec_iters = -1;
   ~mc_batch() {
@@ -1896,6 +1911,10 @@ int batch_create(mc_system *const *sys, int n, const float *const *y, float *con
     return fail(MC_ECUDA);
   }
   b->n = n;
+  for (int k = 0; k < n; ++k) {
+    b->tiles_fwd = b->tiles_fwd || hs[k].warp_fwd;
+    b->tiles_bwd = b->tiles_bwd || hs[k].warp_bwd;
+  }
   b->n_tiles_fwd = tf[n];
   b->n_tiles_bwd = tb[n];
   *out = b;
@@ -1916,11 +1935,13 @@ static int batch_enqueue(mc_batch *b, int n_iter, cudaStream_t s) {
   for (int it = 0; it < n_iter; ++it) {
     if (b->n_tiles_fwd) {
       count_launch();
-      launch_pdl(batch_forward_kernel, (unsigned)b->n_tiles_fwd, kStreamThreads, s, sys, b->tile_fwd.as<uint64_t>(), b->n);
+      launch_pdl(b->tiles_fwd ? batch_forward_kernel<true> : batch_forward_kernel<false>, (unsigned)b->n_tiles_fwd,
+                 kStreamThreads, s, sys, (const uint64_t *)b->tile_fwd.as<uint64_t>(), b->n);
     }
     if (b->n_tiles_bwd) {
       count_launch();
-      launch_pdl(batch_back_kernel, (unsigned)b->n_tiles_bwd, kStreamThreads, s, sys, b->tile_bwd.as<uint64_t>(), b->n);
+      launch_pdl(b->tiles_bwd ? batch_back_kernel<true> : batch_back_kernel<false>, (unsigned)b->n_tiles_bwd,
+                 kStreamThreads, s, sys, (const uint64_t *)b->tile_bwd.as<uint64_t>(), b->n);
     }
   }
   count_launch();

@@ -47,3 +47,25 @@ def test_tiles_match_oracle(mc, m, n, row_len, used, long):
     mc.mlem_iterate(s, torch.as_tensor(y).cuda(), xd, 5)
     want = oracle.mlem(a, y, x0, 5)
     assert np.linalg.norm(xd.cpu().numpy() - want) <= 1e-5 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("lens", [[(1, 2)], [(18, 30)], [(1, 2), (18, 30), (1, 6)]])
+def test_batches_with_and_without_tiles(mc, lens):
+    """The batch kernels of batches whose systems are all warp chunks, all
+    tiles, or mixed, against the oracle."""
+    import torch
+    sysm, ys, xs, want = [], [], [], []
+    for i, rl in enumerate(lens):
+        m, n = 3000 + 7 * i, 1100 + i
+        rows, cols = P.random_events(m, n, rl, 2, 20 + i)
+        sysm.append(mc.mc_system_from_events(m, n, rows, cols, 0, 2 * n))
+        a = oracle.system_matrix(oracle.system_counts(rows, cols, m, n), oracle.histories_per_voxel(n, 0, 2 * n))
+        y = P.poisson_counts(a @ np.linspace(1, 2, n), 20.0 * m, i)
+        ys.append(torch.as_tensor(y).cuda())
+        xs.append(torch.empty(n, dtype=torch.float32, device="cuda"))
+        want.append(oracle.mlem(a, y, oracle.mlem_init(a, y), 6))
+    b = mc.mc_batch_create(sysm, ys, xs)
+    for run in (mc.mc_batch_mlem, mc.mc_batch_mlem_persistent):
+        run(b, 6)
+        for x, w in zip(xs, want):
+            assert np.linalg.norm(x.cpu().numpy() - w) <= 1e-5 * np.linalg.norm(w)
