@@ -295,6 +295,8 @@ static int prepare_plan(const mc_phantom *ph, const mc_geometry *g, cudaStream_t
     count_launch();
     pack_cubes_kernel<<<(int)g, 256, 0, s>>>(ts.material_dev, skip.as<uint8_t>(), (int64_t)nv, pl.cubes.as<uint16_t>());
     MCS_LAUNCHED();
+    // the plan may be built on another stream: the map is complete on return
+    MCS_CUDA(cudaStreamSynchronize(s));
     ts.cubes_dev = pl.cubes.as<uint16_t>();
   }
   return MC_OK;
