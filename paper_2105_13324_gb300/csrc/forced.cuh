@@ -170,10 +170,12 @@ __device__ __forceinline__ int small_int(float k) { return __float_as_int(k + 83
 // own next face on one axis, so mu times the length up to there is the exact
 // integral over the cube (D = 1 is one ordinary voxel step).  Returns whether
 // the ray has left the grid.  Every step that does not crosses at least one face
-// outward on one axis, so a ray ends after nx + ny + nz steps at most.
+// outward on one axis -- a distance of 0 counts as 1, and a ray without a
+// next face before the exit (or with a NaN there) ends -- so a ray ends after
+// nx + ny + nz steps at most, whatever the map and the ray hold.
 __device__ __forceinline__ bool ray_step(const TArgs<float> &a, const float2 *s_mu, Ray &r) {
   const uint32_t cell = __ldg(a.cubes + (uint32_t)((r.iz * a.ny + r.iy) * a.nx + r.ix));
-  const float D = __uint_as_float(0x4B000000u | cell >> 8) - 8388608.0f;
+  const float D = fmaxf(__uint_as_float(0x4B000000u | cell >> 8) - 8388608.0f, 1.0f);
   const float2 c = s_mu[cell & 255u];
   const float e = D - 1.0f;
   const float cx = fmaf(e, r.dtx, r.tx), cy = fmaf(e, r.dty, r.ty), cz = fmaf(e, r.dtz, r.tz);
@@ -188,7 +190,7 @@ __device__ __forceinline__ bool ray_step(const TArgs<float> &a, const float2 *s_
   r.tx = fmaf(kx, r.dtx, r.tx);
   r.ty = fmaf(ky, r.dty, r.ty);
   r.tz = fmaf(kz, r.dtz, r.tz);
-  return tc >= r.t_grid || (unsigned)r.ix >= (unsigned)a.nx || (unsigned)r.iy >= (unsigned)a.ny ||
+  return !(tc < r.t_grid) || (unsigned)r.ix >= (unsigned)a.nx || (unsigned)r.iy >= (unsigned)a.ny ||
          (unsigned)r.iz >= (unsigned)a.nz;
 }
 
