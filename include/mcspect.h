@@ -426,8 +426,9 @@ MC_API int mc_batch_free(mc_batch *batch);
  * memory: a reconstruction service that plans its memory up front (a device
  * allocation or free can synchronise the whole device and stall concurrent
  * work, or fail under a fixed memory cap), or host code whose device memory
- * is owned by another allocator.  mlem_iterate may allocate its
- * log-likelihood buffer on first use; this entry point never calls
+ * is owned by another allocator.  mlem_iterate with likelihoods
+ * allocates its log-likelihood buffer on first use, and up to 64 MB for the
+ * length of a call, from the stream's pool; this entry point never calls
  * cudaMalloc, cudaFree or any allocating routine.  The paper has no
  * counterpart: it is a deployment variant of the ML-EM update above.
  *

@@ -1085,14 +1085,28 @@ static int em_loop(const mc_system *sys, const float *y, float *x, float *xs, fl
 }
 
 int mlem_run(mc_system *sys, const float *y, float *x, int n_iter, bool want_ll, cudaStream_t s) {
+  // Room for the partials of all iterations, up to 64 MB, for this call alone
+  // and in its stream's order: the system's own block may still be in use by
+  // calls queued before, on another stream than the one it was made on.  Where
+  // the room is refused, the system's block does, an iteration at a time.
+  DevBuf group;
+  double *partials = sys->partials.as<double>();
+  int64_t room = (int64_t)(sys->partials.bytes / sizeof(double));
   if (want_ll) {
-    // room for the partials of all iterations, up to 64 MB
     const int64_t fb = forward_blocks(sys);
     const int64_t want = std::min<int64_t>(fb * n_iter, std::max<int64_t>(fb, (64 << 20) / 8));
-    if ((int64_t)(sys->partials.bytes / sizeof(double)) < want) MCS_TRY(sys->partials.alloc((size_t)want * sizeof(double), s));
+    if (room < want) {
+      if (group.alloc((size_t)want * sizeof(double), s) == MC_OK) {
+        partials = group.as<double>();
+        room = want;
+      } else {
+        (void)cudaGetLastError();
+        clear_error();
+      }
+    }
   }
-  return em_loop(sys, y, x, sys->xs.as<float>(), sys->r.as<float>(), sys->partials.as<double>(),
-                 (int64_t)(sys->partials.bytes / sizeof(double)), want_ll ? sys->ll.as<double>() : nullptr, n_iter, s);
+  return em_loop(sys, y, x, sys->xs.as<float>(), sys->r.as<float>(), partials, room,
+                 want_ll ? sys->ll.as<double>() : nullptr, n_iter, s);
 }
 
 }  // namespace mcs
