@@ -864,6 +864,38 @@ static int stream_tiles(const DevBuf &ptr, int64_t n, int64_t nnz, DevBuf &tiles
   return MC_OK;
 }
 
+// The projector layout of a system, to go back to on an error.
+struct Layout {
+  int64_t fwd_blocks, bwd_blocks;
+  int fwd_group, bwd_group;
+  bool fwd_warp, bwd_warp;
+  explicit Layout(const mc_system *s)
+      : fwd_blocks(s->n_csr_blocks), bwd_blocks(s->n_csc_blocks), fwd_group(s->spmv_group_fwd),
+        bwd_group(s->spmv_group_bwd), fwd_warp(s->warp_rows_fwd), bwd_warp(s->warp_rows_bwd) {}
+  void restore(mc_system *s) const {
+    s->n_csr_blocks = fwd_blocks; s->n_csc_blocks = bwd_blocks;
+    s->spmv_group_fwd = fwd_group; s->spmv_group_bwd = bwd_group;
+    s->warp_rows_fwd = fwd_warp; s->warp_rows_bwd = bwd_warp;
+  }
+};
+
+// Makes the log-likelihood partials cover the forward blocks of the present
+// layout, and waits for the stream.  The old block goes only then: calls queued
+// before may still write to it, and it goes back to the pool in the order of
+// the stream that made it, which need not be this one.  Where the room is
+// refused the system returns to layout `old`, which its block covers.
+static int reserve_partials(mc_system *sys, const Layout &old, cudaStream_t s) {
+  const size_t need = (size_t)forward_blocks(sys) * sizeof(double);
+  DevBuf fresh;
+  if (need > sys->partials.bytes) {
+    const int rc = fresh.alloc(need, s);
+    if (rc != MC_OK) { old.restore(sys); return rc; }
+  }
+  MCS_CUDA(cudaStreamSynchronize(s));
+  if (fresh.p) sys->partials = std::move(fresh);
+  return MC_OK;
+}
+
 // Forced projector layouts (mc_system_set_spmv_layout): 0 = streaming
 // tiles (made now if the system has none), 1..32 = lanes per row group,
 // -1 = keep.  On an error the system keeps its previous layout.
@@ -873,6 +905,7 @@ int set_spmv_layout(mc_system *sys, int fwd, int bwd, cudaStream_t s) {
     set_error("layouts must be -1 (keep), 0 (streaming tiles) or 1, 2, 4, 8, 16, 32 lanes; got %d, %d", fwd, bwd);
     return MC_EINVAL;
   }
+  const Layout old(sys);
   DevBuf ft, bt;
   int64_t nft = 0, nbt = 0;
   bool fw = sys->warp_rows_fwd, bw = sys->warp_rows_bwd;
@@ -884,11 +917,7 @@ int set_spmv_layout(mc_system *sys, int fwd, int bwd, cudaStream_t s) {
   if (bwd == 0 && sys->n_csc_blocks == 0) { sys->csc_blocks = std::move(bt); sys->n_csc_blocks = nbt; sys->warp_rows_bwd = bw; }
   if (fwd > 0) { sys->n_csr_blocks = 0; sys->spmv_group_fwd = fwd; }
   if (bwd > 0) { sys->n_csc_blocks = 0; sys->spmv_group_bwd = bwd; }
-  // the log-likelihood partials must cover the forward blocks of the layout
-  const int fb = forward_blocks(sys);
-  if ((size_t)fb * sizeof(double) > sys->partials.bytes) MCS_TRY(sys->partials.alloc((size_t)fb * sizeof(double), s));
-  MCS_CUDA(cudaStreamSynchronize(s));
-  return MC_OK;
+  return reserve_partials(sys, old, s);
 }
 
 int make_stream_blocks(mc_system *sys, cudaStream_t s) {
@@ -2039,6 +2068,7 @@ int autotune(mc_system *sys, cudaStream_t s, int *fwd_choice, int *bwd_choice) {
   cudaEvent_t a = nullptr, b = nullptr;
   MCS_CUDA(cudaEventCreate(&a));
   MCS_CUDA(cudaEventCreate(&b));
+  const Layout old(sys);
   const int64_t fwd_tiles = sys->n_csr_blocks, bwd_tiles = sys->n_csc_blocks;
   const int g_fwd0 = sys->spmv_group_fwd, g_bwd0 = sys->spmv_group_bwd;
   float best_f = 1e30f, best_b = 1e30f;
@@ -2076,12 +2106,9 @@ int autotune(mc_system *sys, cudaStream_t s, int *fwd_choice, int *bwd_choice) {
   sys->n_csc_blocks = choice_b == -1 ? bwd_tiles : 0;
   sys->spmv_group_fwd = choice_f >= 0 ? groups[choice_f] : g_fwd0;
   sys->spmv_group_bwd = choice_b >= 0 ? groups[choice_b] : g_bwd0;
-  // partials must cover the forward blocks of the chosen kernel
-  const int fb = forward_blocks(sys);
-  if ((size_t)fb * sizeof(double) > sys->partials.bytes) MCS_TRY(sys->partials.alloc((size_t)fb * sizeof(double), s));
+  MCS_TRY(reserve_partials(sys, old, s));
   *fwd_choice = choice_f == -1 ? 0 : groups[choice_f];
   *bwd_choice = choice_b == -1 ? 0 : groups[choice_b];
-  MCS_CUDA(cudaStreamSynchronize(s));
   return MC_OK;
 }
 

@@ -91,3 +91,29 @@ def test_with_a_likelihood_queued_before(mc):
     finally:
         stop.set()
         th.join()
+
+
+def test_layout_change_behind_a_queued_likelihood(mc):
+    """A layout with more forward blocks than the system's partial sums cover,
+    set on the stream that still has a likelihood to do."""
+    import torch
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for change in (lambda s: mc.mc_system_set_spmv_layout(s, 32, 32, stream=b), lambda s: mc.mc_system_autotune(s, stream=b)):
+        s, y, x = _system(mc, stream=a)
+        ref, _, _ = _system(mc)
+        v = [torch.zeros(1, dtype=torch.float64, device="cuda") for _ in range(3)]
+        mc.mc_loglik(ref, x, y, v[0])
+        torch.cuda.synchronize()
+        with torch.cuda.stream(b):
+            torch.cuda._sleep(5_000_000)
+            mc.mc_loglik(s, x, y, v[1], stream=b)
+            change(s)
+            others = [_system(mc, 9000, 500, stream=a)[0] for _ in range(3)]
+            mc.mc_loglik(s, x, y, v[2], stream=b)
+        torch.cuda.synchronize()
+        for t in others:
+            t.free()
+        assert v[1].item() == v[0].item()
+        # another layout adds the rows' FP32 sums in another order: 1e-6 of the terms
+        assert abs(v[2].item() - v[0].item()) <= 1e-6 * y.sum().item() * 10
