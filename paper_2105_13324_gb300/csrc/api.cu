@@ -1036,6 +1036,7 @@ int mlem_iterate(mc_system *sys, const float *y_dev, float *x_dev, int32_t n_ite
   cudaStream_t s = API_STREAM(stream);
   const bool want = loglik_host != nullptr && n_iter > 0;
   if (want && sys->ll_cap < n_iter) {
+    sys->ll_cap = 0;  // a refused allocation leaves no buffer
     MCS_TRY(sys->ll.alloc((size_t)n_iter * sizeof(double), s));
     sys->ll_cap = n_iter;
   }
