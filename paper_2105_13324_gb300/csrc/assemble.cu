@@ -1482,6 +1482,10 @@ static int assemble_radix(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t 
 
 int assemble_system(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t s, DevBuf *weights) {
   const uint64_t N = (uint64_t)sys->n_cols;
+  if (n >= 0xFFFFFFFFll) {  // places are 32-bit on every path below
+    set_error("%lld events exceed the 2^32 limit of one build; split the history range", (long long)n);
+    return MC_EINVAL;
+  }
   // n_v and 1/n_v
   MCS_TRY(sys->n_v.alloc(N * sizeof(uint32_t), s));
   MCS_TRY(sys->inv_n.alloc(N * sizeof(float), s));
