@@ -36,20 +36,66 @@ __global__ void prescale_kernel(const float *x, const float *inv_n, float *xs, i
     xs[i] = x[i] * inv_n[i];
 }
 
-// ln q in FP64 for a float q > 0, for the log-likelihood: the FP64 unit issues
-// about two operations per clock and SM, and the library's log (some forty of
-// them) took four fifths of the forward projection that evaluates one per
-// bin.  Here q = 2^e m, m in [sqrt(1/2), sqrt(2)), and with c = 1/m to 24 bits at
-// the middle of m's interval of 2^14 units in the last place, r = m c - 1 is
-// exact (48 bits) and |r| < 2^-9.9:
-//   ln q = e ln 2 - ln c + (r - r^2/2 + r^3/3 - r^4/4 + r^5/5),
-// the omitted term below 2^-61: ten FP64 operations, within 0.6 units in the
-// last place of ln q away from 1 and 2^-58 near it.
-// The table is the definition evaluated at compile time, ln c by the atanh
-// series.
-constexpr int kLogBits = 9;
-constexpr uint32_t kLogFirst = 0x3F3504F3u;  // the float at sqrt(1/2)
-struct alignas(16) LogEntry { double c, l; };
+// A float as a double, from its bits: a conversion instruction runs on the FP64
+// unit, which issues about two operations per clock and SM.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
+  if (a - 0x00800000u >= 0x7F000000u && a != 0u) return (double)x;  // denormal, infinite, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+}
+
+// ... of a normal float, which needs no test
+__device__ __forceinline__ double widen_normal(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// ln q in FP64 for a float q > 0, for the log-likelihood: the library's log
+// (some forty FP64 operations) took most of the forward projection that
+// evaluates one per bin.  Table-driven reduction (P. T. P. Tang, ACM Trans.
+// Math. Softw. 16, 1990): q = 2^e m, m in [0.7067, 1.4135), and with c = 1/m to
+// 24 bits at the middle of m's interval of 2^13 units in the last place, r =
+// m c - 1 is exact (48 bits) and |r| < 2^-11:
+//   ln q = e ln 2 - ln c + (r - r^2/2 + r^3/3 - r^4 (1/4 - r/5 + r^2/6)),
+// the omitted term below 2^-79.  The high parts of ln 2 and -ln c are multiples
+// of 2^-45, so that w = e ln 2 - ln c is exact in them, w + r is split into its
+// rounded sum and the rest, and the low parts join the rest.  The interval
+// around 1 has c = 1 and w = 0.  What stays below 2^-70 of ln q's size near 1
+// (the bracket, the low parts) is formed in float: twelve FP64 operations.
+// Against extended-precision logarithms of every float in (1/2, 2) and 3e7
+// others: 0.515 units in the last place at most (the library's: 0.509 on the
+// test's values).  mc_loglik on the 128^3, 7.3e6-entry matrix: 174 us with the
+// library's log, 109 with this one.
+constexpr int kLogBits = 10;
+constexpr uint32_t kLogFirst = 0x3F34EAABu;  // 1 lies near the middle of an interval
+constexpr double kLn2Hi = 0x1.62e42fefa3ap-1, kLn2Lo = -1.8641886737243033e-15;  // the former a multiple of 2^-45
+struct alignas(16) LogEntry { float c, lo; double hi; };  // c, -ln c = hi + lo
+// Two doubles as an unevaluated sum, at compile time (Dekker 1971).
+struct Pair {
+  double h, l;
+  static constexpr Pair sum(double a, double b) {
+    const double s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+  }
+  static constexpr Pair prod(double a, double b) {
+    const double p = a * b, ca = 134217729.0 * a, cb = 134217729.0 * b;
+    const double ah = ca - (ca - a), bh = cb - (cb - b), al = a - ah, bl = b - bh;
+    return {p, ((ah * bh - p) + ah * bl + al * bh) + al * bl};
+  }
+  constexpr Pair operator+(Pair o) const {
+    const Pair s = sum(h, o.h);
+    return sum(s.h, s.l + (l + o.l));
+  }
+  constexpr Pair operator*(Pair o) const {
+    const Pair p = prod(h, o.h);
+    return sum(p.h, p.l + (h * o.l + l * o.h));
+  }
+  static constexpr Pair quotient(double a, double b) {
+    const double q = a / b;
+    const Pair p = prod(q, b);
+    return sum(q, ((a - p.h) - p.l) / b);
+  }
+};
 struct LogTable {
   LogEntry t[1 << kLogBits];
   static constexpr double value(uint32_t bits) {  // of a float in [1/2, 2)
@@ -58,14 +104,19 @@ struct LogTable {
   }
   constexpr LogTable() : t() {
     for (uint32_t i = 0; i < (1u << kLogBits); ++i) {
-      const uint32_t lo = kLogFirst + (i << (23 - kLogBits));
-      const float c = (float)(2.0 / (value(lo) + value(lo + (1u << (23 - kLogBits)))));
-      // ln c = 2 atanh z, z = (c - 1) / (c + 1), |z| < 0.18, smallest terms first
-      const double z = ((double)c - 1.0) / ((double)c + 1.0), z2 = z * z;
-      double s = 0.0;
-      for (int k = 25; k >= 3; k -= 2) s = (s + 1.0 / k) * z2;
-      t[i].c = (double)c;
-      t[i].l = -2.0 * (z + z * s);
+      const uint32_t a = kLogFirst + (i << (23 - kLogBits)), b = a + (1u << (23 - kLogBits));
+      const float c = a <= 0x3F800000u && b > 0x3F800000u ? 1.0f : (float)(2.0 / (value(a) + value(b)));
+      // -ln c = -2 atanh z, z = (c - 1) / (c + 1), |z| < 0.18: the terms from
+      // z^9 on need no more than a double
+      const Pair z = Pair::quotient((double)c - 1.0, (double)c + 1.0), z2 = z * z;
+      double tail = 0.0;
+      for (int k = 33; k >= 9; k -= 2) tail = tail * z2.h + 1.0 / k;
+      Pair s = {tail, 0.0};
+      for (int k = 7; k >= 1; k -= 2) s = s * z2 + Pair::quotient(1.0, k);
+      const Pair l = z * s * Pair{-2.0, 0.0};
+      t[i].c = c;
+      t[i].hi = (l.h + 192.0) - 192.0;  // rounded to a multiple of 2^-45
+      t[i].lo = (float)((l.h - t[i].hi) + l.l);
     }
   }
 };
@@ -75,19 +126,18 @@ __device__ __forceinline__ double log_of(float q) {
   const uint32_t b = __float_as_uint(q);
   if (b - 0x00800000u >= 0x7F000000u) return log((double)q);  // zero, denormal, infinite, NaN, negative
   const uint32_t d = b - kLogFirst;
-  const double2 t = __ldg(reinterpret_cast<const double2 *>(g_log.t) + (d >> (23 - kLogBits) & ((1u << kLogBits) - 1u)));
+  const uint4 t = __ldg(reinterpret_cast<const uint4 *>(g_log.t) + (d >> (23 - kLogBits) & ((1u << kLogBits) - 1u)));
   const int e = (int)d >> 23;
-  const uint32_t mb = b - ((uint32_t)e << 23);  // m's bits
-  // m and e as doubles, from their bits
-  const double m = __hiloint2double((int)((mb >> 3) + 0x38000000u), (int)(mb << 29));
-  const double x = __hiloint2double(0x43380000, e + 256) - 6755399441056000.0;  // 1.5 2^52 + 256
-  const double r = fma(m, t.x, -1.0);
-  double p = fma(r, 0.2, -0.25);
-  p = fma(p, r, 1.0 / 3.0);
-  p = fma(p, r, -0.5);
-  // ln 2 = hi (40 bits, x hi is exact) + lo: one rounding at the size of ln q
-  p = fma(p, r * r, r) + fma(x, 7.3710025651677989018e-13, t.y);
-  return fma(x, 0.6931471805592082091607153, p);
+  const float mf = __uint_as_float(b - ((uint32_t)e << 23)), cf = __uint_as_float(t.x);
+  const double x = __hiloint2double(0x43380000, e + 256) - 6755399441056000.0;  // e: 1.5 2^52 + 256
+  const double r = fma(widen_normal(mf), widen_normal(cf), -1.0);
+  const float rf = fmaf(mf, cf, -1.0f);
+  const float p = fmaf(-rf, fmaf(rf, -1.0f / 6.0f, 0.2f), 0.25f);
+  const double s = fma(fma(-widen_normal(p), r, 1.0 / 3.0), r, -0.5);
+  const double w = fma(x, kLn2Hi, __hiloint2double((int)t.w, (int)t.z));
+  const double hi = w + r;
+  const float low = fmaf((float)e, (float)kLn2Lo, __uint_as_float(t.y));  // 0 (at e = 0, c = 1) or normal
+  return hi + fma(s, r * r, ((w - hi) + r) + (low == 0.0f ? 0.0 : widen_normal(low)));
 }
 
 // Sum of a double over the block (fixed order); valid in thread 0.
@@ -214,7 +264,7 @@ __global__ void __launch_bounds__(kSpmvThreads) csr_forward_kernel(const uint32_
         // a bin with an empty row is left out of the y ln q sum (q = 0 for
         // every image: the term carries no information about x)
         const float yj = MODE == 1 ? yv : y[gid];
-        ll = (yj > 0.0f && e > b ? (double)yj * log_of(acc) : 0.0) - (double)acc;
+        ll = (yj > 0.0f && e > b ? widen(yj) * log_of(acc) : 0.0) - widen(acc);
       }
     }
   }
@@ -438,7 +488,7 @@ struct FwdOut {
       out[r] = acc;
     } else if (MODE == 1) {
       out[r] = acc > 0.0f ? yv / acc : 0.0f;
-      if (LL) ll += (yv > 0.0f && reached ? (double)yv * log_of(acc) : 0.0) - (double)acc;
+      if (LL) ll += (yv > 0.0f && reached ? widen(yv) * log_of(acc) : 0.0) - widen(acc);
     } else {
       out[r] = ratio_out<MODE>(acc, r, y, rmap, add);
     }
