@@ -1314,23 +1314,25 @@ __global__ void back_f64_kernel(const uint32_t *col_ptr, const uint32_t *row, co
 }
 
 // The float prior and the gradient step are bound by the FP64 unit when they
-// compute in double (about two operations per clock and SM; conversions count).
-// Both have float inputs and outputs, so they run on unevaluated sums of two
-// floats instead (Dekker 1971, Knuth's two-sum): exact differences and products,
-// about 45 bits in the sums, rounded once to float at the end.  Voxels whose
-// values leave the range where that holds take the double formulas.  Against
-// 64 bits the results' errors are those of the double kernels (the final
-// rounding).  128^3 on a GB300: the step 73 -> 14 us, the prior's value 56 -> 24, its
-// gradient 56 -> 17.
+// compute in double (about two operations per clock and SM).  Both have float
+// inputs, so they run on unevaluated sums of floats instead (Dekker 1971,
+// Knuth's two-sum): exact differences and products; two floats, about 45 bits,
+// in the sums that are rounded to float at the end, three floats in the
+// value's, which stays an FP64 result.  Voxels whose values leave the range
+// where that holds take the double formulas.  128^3 on a GB300: the step 109 ->
+// 12 us a call, the prior's value 60 -> 30, its gradient 99 -> 17, both 115 -> 37.
 struct Two { float h, l; };
+// (every rounding is meant: a product fused into one of these sums would be
+// counted twice)
 __device__ __forceinline__ Two two_sum(float a, float b) {
-  const float s = a + b, t = s - a;
-  return {s, (a - (s - t)) + (b - t)};
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
 }
 __device__ __forceinline__ Two two_diff(float a, float b) { return two_sum(a, -b); }
 __device__ __forceinline__ bool in_range(float x, float lo, float hi) { return fabsf(x) >= lo && fabsf(x) <= hi; }
-constexpr float kTwoM80 = 8.2718061255302767e-25f, kTwoM60 = 8.6736173798840355e-19f, kTwoM50 = 8.8817841970012523e-16f,
-                kTwoM40 = 9.0949470177292824e-13f, kTwoM16 = 1.52587890625e-05f, kTwo60 = 1.152921504606846976e18f;
+constexpr float kTwoM80 = 8.2718061255302767e-25f, kTwoM60 = 8.6736173798840355e-19f,
+                kTwoM40 = 9.0949470177292824e-13f, kTwoM16 = 1.52587890625e-05f, kTwo20 = 1048576.0f,
+                kTwo30 = 1073741824.0f, kTwo60 = 1.152921504606846976e18f;
 
 // the prior's terms at one voxel, in double
 template <typename T>
@@ -1365,6 +1367,29 @@ __global__ void prior_kernel(int nx, int ny, int nz, double beta, const T *x, T 
   }
 }
 
+// A sum of squares as an unevaluated sum of three floats: an FP64 sum of the
+// 53-bit squares costs six FP64 operations a voxel (56 us at 128^3 against 30).
+// add() takes the square of the exact difference d, times 2^40 so that small
+// differences keep their low parts: h^2 = p + e and 2 h l = q + f exactly, and
+// l^2.  What is rounded are the third float's sums, 2^-24 of terms below 2^-44 of
+// the whole.
+struct Three {
+  float a, b, c;
+  __device__ __forceinline__ void add(Two d) {
+    const float h = d.h * kTwo20, l = d.l * kTwo20, h2 = 2.0f * h;
+    const float p = __fmul_rn(h, h), e = fmaf(h, h, -p), q = __fmul_rn(h2, l), f = fmaf(h2, l, -q);
+    const Two s = two_sum(a, p), t = two_sum(b, s.l), u = two_sum(t.h, e), w = two_sum(u.h, q);
+    a = s.h;
+    b = w.h;
+    c += (t.l + u.l) + (w.l + fmaf(l, l, f));
+  }
+  __device__ __forceinline__ void normalise() {
+    const Two s = two_sum(a, b), t = two_sum(s.l, c);
+    a = s.h; b = t.h; c = t.l;
+  }
+  __device__ __forceinline__ double value() const { return ((double)a + ((double)b + (double)c)) * 0x1p-40; }
+};
+
 // prior_kernel for float images of fewer than 2^31 voxels and 2^-40 <= beta <=
 // 2^40 (bh + bl)
 template <bool GRAD, bool VALUE>
@@ -1373,7 +1398,7 @@ __global__ void prior_f32_kernel(int nx, int ny, int nz, uint32_t magic_xy, uint
   __shared__ double s_tmp[32];
   const uint32_t n = (uint32_t)nx * ny * nz, nxy = (uint32_t)nx * ny;
   double val = 0.0;
-  Two sum = {0.0f, 0.0f};
+  Three sum = {0.0f, 0.0f, 0.0f};
   for (uint64_t v64 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v64 < n; v64 += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t v = (uint32_t)v64;
     uint32_t r, i;
@@ -1382,8 +1407,6 @@ __global__ void prior_f32_kernel(int nx, int ny, int nz, uint32_t magic_xy, uint
     // a missing neighbour counts as an equal one
     const Two d[3] = {two_diff(xv, (int)i < nx - 1 ? x[v + 1] : xv), two_diff(xv, (int)j < ny - 1 ? x[v + nx] : xv),
                       two_diff(xv, (int)k < nz - 1 ? x[v + nxy] : xv)};
-    bool ok = true;
-    float gout = 0.0f;
     if (GRAD) {
       const Two e[3] = {two_diff(xv, i > 0 ? x[v - 1] : xv), two_diff(xv, j > 0 ? x[v - nx] : xv),
                         two_diff(xv, k > 0 ? x[v - nxy] : xv)};
@@ -1396,37 +1419,31 @@ __global__ void prior_f32_kernel(int nx, int ny, int nz, uint32_t magic_xy, uint
         dm = fmaxf(dm, fabsf(a.h));
       }
       const float p = bh * g.h;
-      gout = p + (fmaf(bh, g.h, -p) + (bh * g.l + bl * g.h));
+      float gout = p + (fmaf(bh, g.h, -p) + (bh * g.l + bl * g.h));
       // (a sum that has lost more than 16 bits to cancellation: in double)
-      ok = dm == 0.0f ? g.h == 0.0f : in_range(g.h, fmaxf(kTwoM40, kTwoM16 * dm), kTwo60);
+      if (!(dm == 0.0f ? g.h == 0.0f : in_range(g.h, fmaxf(kTwoM40, kTwoM16 * dm), kTwo60))) {
+        double g64, unused = 0.0;
+        prior_voxel<float>(x, v, (int)i, (int)j, (int)k, nx, ny, nz, g64, unused);
+        gout = (float)(beta * g64);
+      }
+      grad[v] = gout;
     }
-    Two sq = {0.0f, 0.0f};
     if (VALUE) {
       const float m = fmaxf(fmaxf(fabsf(d[0].h), fabsf(d[1].h)), fabsf(d[2].h));
       // (a NaN or infinite difference fails the comparison of the sum)
-      ok = ok && (m == 0.0f ? d[0].h + d[1].h + d[2].h == 0.0f : in_range(m, kTwoM50, 1.0e9f));
+      const float all = d[0].h + d[1].h + d[2].h;
+      if (m == 0.0f ? all == 0.0f : in_range(m, kTwoM60, kTwo30) && all - all == 0.0f) {
 #pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        const float p = d[t].h * d[t].h;
-        const Two s = two_sum(sq.h, p);
-        sq = {s.h, sq.l + (s.l + fmaf(2.0f * d[t].h, d[t].l, fmaf(d[t].h, d[t].h, -p)))};
+        for (int t = 0; t < 3; ++t) sum.add(d[t]);
+        sum.normalise();
+      } else {
+        double unused;
+        prior_voxel<float>(x, v, (int)i, (int)j, (int)k, nx, ny, nz, unused, val);
       }
-      ok = ok && sq.h + sq.l < INFINITY;
     }
-    if (ok) {
-      if (VALUE) {
-        const Two s = two_sum(sum.h, sq.h);
-        sum = two_sum(s.h, sum.l + (s.l + sq.l));
-      }
-    } else {
-      double g64;
-      prior_voxel<float>(x, v, (int)i, (int)j, (int)k, nx, ny, nz, g64, val);
-      gout = (float)(beta * g64);
-    }
-    if (GRAD) grad[v] = gout;
   }
   if (VALUE) {
-    const double t = block_sum_double(0.5 * beta * (val + ((double)sum.h + (double)sum.l)), s_tmp);
+    const double t = block_sum_double(0.5 * beta * (val + sum.value()), s_tmp);
     if (threadIdx.x == 0) partials[blockIdx.x] = t;
   }
 }
