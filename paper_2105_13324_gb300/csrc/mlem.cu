@@ -1319,8 +1319,9 @@ __global__ void back_f64_kernel(const uint32_t *col_ptr, const uint32_t *row, co
 // Knuth's two-sum): exact differences and products; two floats, about 45 bits,
 // in the sums that are rounded to float at the end, three floats in the
 // value's, which stays an FP64 result.  Voxels whose values leave the range
-// where that holds take the double formulas.  128^3 on a GB300: the step 109 ->
-// 12 us a call, the prior's value 60 -> 30, its gradient 99 -> 17, both 115 -> 37.
+// where that holds, or whose rounding it leaves open, take the double formulas.
+// 128^3 on a GB300: the step 109 -> 12.6 us a call, the prior's value 60 -> 29,
+// its gradient 99 -> 18, both 115 -> 39.
 struct Two { float h, l; };
 // (every rounding is meant: a product fused into one of these sums would be
 // counted twice)
@@ -1331,8 +1332,17 @@ __device__ __forceinline__ Two two_sum(float a, float b) {
 __device__ __forceinline__ Two two_diff(float a, float b) { return two_sum(a, -b); }
 __device__ __forceinline__ bool in_range(float x, float lo, float hi) { return fabsf(x) >= lo && fabsf(x) <= hi; }
 constexpr float kTwoM80 = 8.2718061255302767e-25f, kTwoM60 = 8.6736173798840355e-19f,
-                kTwoM40 = 9.0949470177292824e-13f, kTwoM16 = 1.52587890625e-05f, kTwo20 = 1048576.0f,
-                kTwo30 = 1073741824.0f, kTwo60 = 1.152921504606846976e18f;
+                kTwoM40 = 9.0949470177292824e-13f, kTwoM38 = 3.637978807091713e-12f, kTwoM16 = 1.52587890625e-05f,
+                kTwo20 = 1048576.0f, kTwo30 = 1073741824.0f, kTwo60 = 1.152921504606846976e18f;
+
+// out = h + l rounded to float.  False where that is not certain for a value
+// within err of the sum: such a result (one in some ten thousand) is formed in
+// double, so that the others are the correctly rounded ones and none is further
+// off than the double formula's.
+__device__ __forceinline__ bool rounds(float h, float l, float err, float &out) {
+  out = __fadd_rn(h, __fadd_rn(l, err));
+  return out == __fadd_rn(h, __fsub_rn(l, err));
+}
 
 // the prior's terms at one voxel, in double
 template <typename T>
@@ -1418,10 +1428,14 @@ __global__ void prior_f32_kernel(int nx, int ny, int nz, uint32_t magic_xy, uint
         g = {s.h, g.l + (s.l + a.l)};
         dm = fmaxf(dm, fabsf(a.h));
       }
-      const float p = bh * g.h;
-      float gout = p + (fmaf(bh, g.h, -p) + (bh * g.l + bl * g.h));
+      // g is within 2^-40.2 dm of the sum, its product with beta within 2^-39.3
+      // bh dm, the additions below included
+      const float p = __fmul_rn(bh, g.h);
+      float gout;
+      bool ok = rounds(p, fmaf(bh, g.h, -p) + fmaf(bh, g.l, bl * g.h), kTwoM38 * (bh * dm), gout);
       // (a sum that has lost more than 16 bits to cancellation: in double)
-      if (!(dm == 0.0f ? g.h == 0.0f : in_range(g.h, fmaxf(kTwoM40, kTwoM16 * dm), kTwo60))) {
+      ok = ok && (dm == 0.0f ? g.h == 0.0f : in_range(g.h, fmaxf(kTwoM40, kTwoM16 * dm), kTwo60));
+      if (!ok) {
         double g64, unused = 0.0;
         prior_voxel<float>(x, v, (int)i, (int)j, (int)k, nx, ny, nz, g64, unused);
         gout = (float)(beta * g64);
@@ -1454,7 +1468,7 @@ __global__ void prior_f32_kernel(int nx, int ny, int nz, uint32_t magic_xy, uint
 __device__ __noinline__ float pgd_voxel(double alpha, double s, float bp, float gp, float x) {
   if (!(s > 0.0)) return 0.0f;
   const double grad = s - (double)bp + (double)gp;
-  const double xn = (double)x - alpha * ((double)x / s) * grad;
+  const double xn = fma(-(alpha * ((double)x / s)), grad, (double)x);
   return (float)(xn > 0.0 ? xn : 0.0);
 }
 
@@ -1477,19 +1491,20 @@ __global__ void pgd_step_kernel(int64_t n, double alpha, Two a, Two c, bool fast
       const float sl = (float)(lo & 0x1FFFFFFFu) * __uint_as_float((uint32_t)(ex - 52 + 127) << 23);
       const Two t = two_diff(b, g);
       const float ri = __frcp_rn(sh);
-      const float q0 = t.h * ri;
+      const float q0 = __fmul_rn(t.h, ri);
       const float q1 = (fmaf(-q0, sh, t.h) + (t.l - q0 * sl)) * ri;
-      const Two u = two_sum(q0, q1);
-      const float p = a.h * u.h;
-      const float pe = fmaf(a.h, u.h, -p) + (a.h * u.l + a.l * u.h);
+      const Two u = two_sum(q0, q1);  // within 2^-42.9 of its size
+      const float p = __fmul_rn(a.h, u.h);
+      const float pe = fmaf(a.h, u.h, -p) + fmaf(a.h, u.l, a.l * u.h);
       const Two w = two_sum(c.h, p);
       const float wl = w.l + (pe + c.l);
-      const float m = xv * w.h;
-      out = m + (fmaf(xv, w.h, -m) + xv * wl);
+      const float m = __fmul_rn(xv, w.h);
+      // within 2^-41.8 x max(p, c), the additions in rounds() included
+      ok = rounds(m, fmaf(xv, w.h, -m) + xv * wl, kTwoM40 * (xv * fmaxf(fabsf(p), fabsf(c.h))), out);
       // a result that has lost more than 16 bits to cancellation, or is too
       // small for the low parts, is formed in double
       ok = (t.h == 0.0f || fabsf(t.h) >= kTwoM60) &&
-           (xv == 0.0f || out <= -kTwoM16 * xv || (out >= kTwoM16 * xv && out >= kTwoM80));
+           (xv == 0.0f || out <= -kTwoM16 * xv || (ok && out >= kTwoM16 * xv && out >= kTwoM80));
       out = out > 0.0f ? out : 0.0f;
     }
     if (!ok) out = pgd_voxel(alpha, s, b, g, xv);
