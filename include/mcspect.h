@@ -286,7 +286,7 @@ MC_API int mc_system_set_value_type(mc_system *sys, int32_t value_type, int32_t 
  * (back-projection, CSC) each 0 = streaming layout (entries of runs of whole
  * rows staged in shared memory, then one fixed-order sum per row: warps of
  * 32 R rows, R = 1, 2 or 4 rows per lane, when rows average fewer than 16
- * entries, else a thread per row in tiles of ~4096 entries), 1, 2, 4, 8,
+ * entries, else a thread or a warp per row in tiles of ~4096 entries), 1, 2, 4, 8,
  * 16 or 32 = that many lanes per row (column), or -1 = keep.  Every layout
  * gives the same sums up to FP32 rounding order.  The streaming layout needs
  * every row (column) shorter than 2048 entries: MC_EINVAL otherwise (the

@@ -138,7 +138,9 @@ struct mc_system {
   // fall back to the row-group kernels)
   mcs::DevBuf csr_blocks, csc_blocks;  // u32 [n_blocks + 1] first row / column of each tile
   int64_t n_csr_blocks = 0, n_csc_blocks = 0;
-  bool warp_rows_fwd = false, warp_rows_bwd = false;
+  // how the streaming layout sums rows / columns: kChunks, kByThread or
+  // kByThreadOrWarp (mlem.cu)
+  int sums_fwd = 0, sums_bwd = 0;
   // forced detection: the entries are summed event weights instead of
   // counts, in fixed point (q * 2^-48); the counts above are then the
   // number of weighted events per entry

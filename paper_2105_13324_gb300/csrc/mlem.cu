@@ -377,9 +377,9 @@ __global__ void sensitivity_kernel(const double *colsum, const uint32_t *n_v, in
 // CSR (CSC) arrays.  The block first reads the tile's entries and gathers the
 // vector with independent, coalesced loads (many requests in flight), keeps
 // the products in shared memory, and then reduces each row from shared
-// memory, a thread per row.  Segments of fewer than 16 entries on average use
-// the warp chunks below instead.  Every row is summed in a fixed order, so
-// results are reproducible.
+// memory, a thread or a warp per row.  Segments of fewer than 16 entries on
+// average use the warp chunks below instead.  Every row is summed in a fixed
+// order, so results are reproducible.
 constexpr int kStreamTile = 4096;
 constexpr int kStreamThreads = 256;
 
@@ -437,37 +437,65 @@ __device__ __forceinline__ float strided_tree(const float *s_prod, uint32_t b, u
   return a[0];
 }
 
-// Reduces every segment j in [j0, j1) of the tile from shared memory, a thread
-// each, and hands its sum to out.store(j, acc, out.load(j), segment j
-// non-empty).  (A warp per segment, the former reduction, was a chain of five
-// shuffles and a dependent pointer load per segment for 17 to 26 segments one
-// after another: at rows of 18 entries on the 128^3 system 0.262 ms a forward
-// projection against 0.168; at 31, 0.336
-// against 0.267.)
-template <typename Out>
-__device__ __forceinline__ void stream_segments(const uint32_t *__restrict__ ptr, uint32_t j0, uint32_t j1,
-                                                uint32_t p0, const float *s_prod, Out &out) {
-  for (uint32_t j = j0 + threadIdx.x; j < j1; j += kStreamThreads) {
-    const uint32_t b = ptr[j], e = ptr[j + 1];
-    const typename Out::Pre pre = out.load(j);
-    out.store(j, strided_tree(s_prod, b - p0, e - p0), pre, e > b);
-  }
+// The same sum by a warp (result in every lane)
+__device__ __forceinline__ float warp_tree(const float *s_prod, uint32_t b, uint32_t e) {
+  float acc = 0.0f;
+  for (uint32_t k = b + (threadIdx.x & 31); k < e; k += 32) acc += s_prod[k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
 }
 
-// The same sums by a warp per segment: the batch kernels keep it, whose other
-// path (warp chunks, all serving systems take it) would lose a tenth to the
-// registers of the 16 partial sums.
+// Reduces every segment j in [j0, j1) of the tile from shared memory by a warp
+// each, and hands its sum to out.store(j, acc, out.load(j), segment j non-empty).
+// The batch kernels use nothing else: their other path (warp chunks, all serving
+// systems take it) would lose a tenth to the registers of strided_tree.
 template <typename Out>
 __device__ __forceinline__ void stream_segments_warp(const uint32_t *__restrict__ ptr, uint32_t j0, uint32_t j1,
                                                      uint32_t p0, const float *s_prod, Out &out) {
   for (uint32_t j = j0 + (threadIdx.x >> 5); j < j1; j += kStreamThreads / 32) {
     const uint32_t b = ptr[j], e = ptr[j + 1];
-    float acc = 0.0f;
-    for (uint32_t k = b - p0 + (threadIdx.x & 31); k < e - p0; k += 32) acc += s_prod[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const float acc = warp_tree(s_prod, b - p0, e - p0);
     if ((threadIdx.x & 31) == 0) out.store(j, acc, out.load(j), e > b);
   }
+}
+
+// The same sums by a thread per segment, which leaves no lanes idle on short
+// ones (a warp per segment is a chain of five shuffles and a dependent pointer
+// load for 17 to 26 segments one after another: at rows of 18 entries on the
+// 128^3 system 0.262 ms a forward projection against 0.168; at 31, 0.336 against
+// 0.267).  LONG: the system has segments of more than kLongSegment entries.  A
+// tile of long ones holds too few for its 256 threads, so from a mean of
+// kWarpMean on it goes to a warp each (4e7 entries, forward projection in ms,
+// thread and warp: rows of 64 entries 0.180, 0.189; 100 0.185, 0.177; 300 0.188,
+// 0.159; 1000 0.210, 0.133), and a single long segment is summed by the warp that
+// meets it (1 % of rows of 1500 among rows of 3: 0.161, 0.108).  Where there are
+// none, the plain loop is the better code (back-projection of rows of 18 to 64:
+// 0.176 against 0.184).
+constexpr uint32_t kWarpMean = 80, kLongSegment = 128;
+enum { kChunks = 0, kByThread = 1, kByThreadOrWarp = 2 };  // mc_system::sums_fwd, sums_bwd
+template <bool LONG, typename Out>
+__device__ __forceinline__ void stream_segments(const uint32_t *__restrict__ ptr, uint32_t j0, uint32_t j1,
+                                                uint32_t p0, uint32_t cnt, const float *s_prod, Out &out) {
+  if (LONG && cnt >= kWarpMean * (j1 - j0)) {
+    stream_segments_warp(ptr, j0, j1, p0, s_prod, out);
+    return;
+  }
+  bool lengthy = false;
+  for (uint32_t j = j0 + threadIdx.x; j < j1; j += kStreamThreads) {
+    const uint32_t b = ptr[j], e = ptr[j + 1];
+    const typename Out::Pre pre = out.load(j);
+    if (!LONG || e - b <= kLongSegment) out.store(j, strided_tree(s_prod, b - p0, e - p0), pre, e > b);
+    else lengthy = true;
+  }
+  if (!LONG || !__any_sync(0xffffffffu, lengthy)) return;
+  for (uint32_t base = j0 + (threadIdx.x & ~31u); base < j1; base += kStreamThreads)
+    for (uint32_t j = base; j < min(base + 32u, j1); ++j) {
+      const uint32_t b = ptr[j], e = ptr[j + 1];
+      if (e - b <= kLongSegment) continue;
+      const float acc = warp_tree(s_prod, b - p0, e - p0);
+      if ((threadIdx.x & 31) == 0) out.store(j, acc, out.load(j), true);
+    }
 }
 
 // Forward epilogue: MODE 0 q, MODE 1 ratio (+ log-likelihood share),
@@ -523,7 +551,7 @@ struct BackOut {
   }
 };
 
-template <typename V, int MODE, bool LL>
+template <typename V, int MODE, bool LL, bool LONG>
 __global__ void __launch_bounds__(kStreamThreads) stream_forward_kernel(const uint32_t *__restrict__ row_ptr,
                                                                      const uint32_t *__restrict__ tiles,
                                                                      const uint32_t *__restrict__ col,
@@ -537,18 +565,18 @@ __global__ void __launch_bounds__(kStreamThreads) stream_forward_kernel(const ui
   __shared__ double s_tmp[kStreamThreads / 32];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t r0 = tiles[blockIdx.x], r1 = tiles[blockIdx.x + 1];
-  const uint32_t p0 = row_ptr[r0];
-  stream_products<V>(p0, row_ptr[r1] - p0, col, val, xs, s_prod);
+  const uint32_t p0 = row_ptr[r0], cnt = row_ptr[r1] - p0;
+  stream_products<V>(p0, cnt, col, val, xs, s_prod);
   __syncthreads();
   FwdOut<MODE, LL> o{y, out, rmap, add, 0.0};
-  stream_segments(row_ptr, r0, r1, p0, s_prod, o);
+  stream_segments<LONG>(row_ptr, r0, r1, p0, cnt, s_prod, o);
   if (LL) {
     const double t = block_sum_double(o.ll, s_tmp);
     if (threadIdx.x == 0) partials[blockIdx.x] = t;
   }
 }
 
-template <typename V, int MODE>
+template <typename V, int MODE, bool LONG>
 __global__ void __launch_bounds__(kStreamThreads) stream_back_kernel(const uint32_t *__restrict__ col_ptr,
                                                                   const uint32_t *__restrict__ tiles,
                                                                   const uint32_t *__restrict__ row,
@@ -560,11 +588,11 @@ __global__ void __launch_bounds__(kStreamThreads) stream_back_kernel(const uint3
   __shared__ float s_prod[kStreamTile];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t c0 = tiles[blockIdx.x], c1 = tiles[blockIdx.x + 1];
-  const uint32_t p0 = col_ptr[c0];
-  stream_products<V>(p0, col_ptr[c1] - p0, row, val, r, s_prod);
+  const uint32_t p0 = col_ptr[c0], cnt = col_ptr[c1] - p0;
+  stream_products<V>(p0, cnt, row, val, r, s_prod);
   __syncthreads();
   BackOut<MODE> o{inv_n, inv_colsum, x, xs};
-  stream_segments(col_ptr, c0, c1, p0, s_prod, o);
+  stream_segments<LONG>(col_ptr, c0, c1, p0, cnt, s_prod, o);
 }
 
 // ---------------------------------------------------------------------------
@@ -810,8 +838,9 @@ static void stream_fwd_launch(const mc_system *sys, const float *xs, const float
   const uint32_t *rp = sys->row_ptr.as<uint32_t>(), *t = sys->csr_blocks.as<uint32_t>(), *ci = sys->col_idx.as<uint32_t>();
   const V *val = sys->csr_val.as<V>();
   count_launch();
-  if (sys->warp_rows_fwd)
-    launch_pdl(stream_forward_kernel<V, MODE, LL>, nb, kStreamThreads, s, rp, t, ci, val, xs, y, out, partials, rmap, add);
+  if (sys->sums_fwd != kChunks)
+    launch_pdl(sys->sums_fwd == kByThread ? stream_forward_kernel<V, MODE, LL, false>
+                                          : stream_forward_kernel<V, MODE, LL, true>, nb, kStreamThreads, s, rp, t, ci, val, xs, y, out, partials, rmap, add);
   else {
     const int R = chunk_rows_per_lane(sys->nnz, sys->n_rows, sys->n_rows);
     const unsigned g = (unsigned)div_up(sys->n_rows, (int64_t)kChunkThreads * R);
@@ -830,8 +859,9 @@ static void stream_back_launch(const mc_system *sys, const float *r, float *x, f
   const V *val = sys->csc_val.as<V>();
   const float *inv_n = scale ? scale : proj_scale(sys), *ics = proj_inv_norm(sys);
   count_launch();
-  if (sys->warp_rows_bwd)
-    launch_pdl(stream_back_kernel<V, MODE>, nb, kStreamThreads, s, cp, t, ri, val, r, inv_n, ics, x, xs);
+  if (sys->sums_bwd != kChunks)
+    launch_pdl(sys->sums_bwd == kByThread ? stream_back_kernel<V, MODE, false> : stream_back_kernel<V, MODE, true>, nb,
+               kStreamThreads, s, cp, t, ri, val, r, inv_n, ics, x, xs);
   else {
     const int R = chunk_rows_per_lane(sys->nnz, sys->n_cols, sys->n_cols);
     const unsigned g = (unsigned)div_up(sys->n_cols, (int64_t)kChunkThreads * R);
@@ -874,7 +904,7 @@ static void back_dispatch(const mc_system *sys, const float *r, float *x, float 
 }
 
 int forward_blocks(const mc_system *sys) {
-  if (sys->n_csr_blocks > 0 && !sys->warp_rows_fwd)  // warp chunks
+  if (sys->n_csr_blocks > 0 && sys->sums_fwd == kChunks)
     return div_up(sys->n_rows, (int64_t)kChunkThreads * chunk_rows_per_lane(sys->nnz, sys->n_rows, sys->n_rows));
   if (sys->n_csr_blocks > 0) return (int)sys->n_csr_blocks;
   return div_up(sys->n_rows * sys->spmv_group_fwd, kSpmvThreads);
@@ -883,7 +913,7 @@ int forward_blocks(const mc_system *sys) {
 // Tiles for one pointer array.  Unless `force`, none (row-group kernels)
 // when a segment is longer than half a tile or the mean segment is long;
 // with `force` a segment longer than half a tile is an error.
-static int stream_tiles(const DevBuf &ptr, int64_t n, int64_t nnz, DevBuf &tiles, int64_t &n_tiles, bool &warp,
+static int stream_tiles(const DevBuf &ptr, int64_t n, int64_t nnz, DevBuf &tiles, int64_t &n_tiles, int &sums,
                         cudaStream_t s, bool force = false) {
   n_tiles = 0;
   if (n <= 0 || nnz <= 0) return MC_OK;
@@ -910,22 +940,21 @@ static int stream_tiles(const DevBuf &ptr, int64_t n, int64_t nnz, DevBuf &tiles
   tile_bounds_kernel<<<grid_stride_blocks(n_tiles + 1), 256, 0, s>>>(ptr.as<uint32_t>(), n, step, n_tiles,
                                                                      tiles.as<uint32_t>());
   MCS_LAUNCHED();
-  warp = (double)nnz / (double)n >= 16.0;
+  sums = (double)nnz / (double)n < 16.0 ? kChunks : longest > kLongSegment ? kByThreadOrWarp : kByThread;
   return MC_OK;
 }
 
 // The projector layout of a system, to go back to on an error.
 struct Layout {
   int64_t fwd_blocks, bwd_blocks;
-  int fwd_group, bwd_group;
-  bool fwd_warp, bwd_warp;
+  int fwd_group, bwd_group, fwd_sums, bwd_sums;
   explicit Layout(const mc_system *s)
       : fwd_blocks(s->n_csr_blocks), bwd_blocks(s->n_csc_blocks), fwd_group(s->spmv_group_fwd),
-        bwd_group(s->spmv_group_bwd), fwd_warp(s->warp_rows_fwd), bwd_warp(s->warp_rows_bwd) {}
+        bwd_group(s->spmv_group_bwd), fwd_sums(s->sums_fwd), bwd_sums(s->sums_bwd) {}
   void restore(mc_system *s) const {
     s->n_csr_blocks = fwd_blocks; s->n_csc_blocks = bwd_blocks;
     s->spmv_group_fwd = fwd_group; s->spmv_group_bwd = bwd_group;
-    s->warp_rows_fwd = fwd_warp; s->warp_rows_bwd = bwd_warp;
+    s->sums_fwd = fwd_sums; s->sums_bwd = bwd_sums;
   }
 };
 
@@ -958,21 +987,21 @@ int set_spmv_layout(mc_system *sys, int fwd, int bwd, cudaStream_t s) {
   const Layout old(sys);
   DevBuf ft, bt;
   int64_t nft = 0, nbt = 0;
-  bool fw = sys->warp_rows_fwd, bw = sys->warp_rows_bwd;
+  int fw = sys->sums_fwd, bw = sys->sums_bwd;
   if (fwd == 0 && sys->n_csr_blocks == 0)
     MCS_TRY(stream_tiles(sys->row_ptr, sys->n_rows, sys->nnz, ft, nft, fw, s, true));
   if (bwd == 0 && sys->n_csc_blocks == 0)
     MCS_TRY(stream_tiles(sys->col_ptr, sys->n_cols, sys->nnz, bt, nbt, bw, s, true));
-  if (fwd == 0 && sys->n_csr_blocks == 0) { sys->csr_blocks = std::move(ft); sys->n_csr_blocks = nft; sys->warp_rows_fwd = fw; }
-  if (bwd == 0 && sys->n_csc_blocks == 0) { sys->csc_blocks = std::move(bt); sys->n_csc_blocks = nbt; sys->warp_rows_bwd = bw; }
+  if (fwd == 0 && sys->n_csr_blocks == 0) { sys->csr_blocks = std::move(ft); sys->n_csr_blocks = nft; sys->sums_fwd = fw; }
+  if (bwd == 0 && sys->n_csc_blocks == 0) { sys->csc_blocks = std::move(bt); sys->n_csc_blocks = nbt; sys->sums_bwd = bw; }
   if (fwd > 0) { sys->n_csr_blocks = 0; sys->spmv_group_fwd = fwd; }
   if (bwd > 0) { sys->n_csc_blocks = 0; sys->spmv_group_bwd = bwd; }
   return reserve_partials(sys, old, s);
 }
 
 int make_stream_blocks(mc_system *sys, cudaStream_t s) {
-  MCS_TRY(stream_tiles(sys->row_ptr, sys->n_rows, sys->nnz, sys->csr_blocks, sys->n_csr_blocks, sys->warp_rows_fwd, s));
-  MCS_TRY(stream_tiles(sys->col_ptr, sys->n_cols, sys->nnz, sys->csc_blocks, sys->n_csc_blocks, sys->warp_rows_bwd, s));
+  MCS_TRY(stream_tiles(sys->row_ptr, sys->n_rows, sys->nnz, sys->csr_blocks, sys->n_csr_blocks, sys->sums_fwd, s));
+  MCS_TRY(stream_tiles(sys->col_ptr, sys->n_cols, sys->nnz, sys->csc_blocks, sys->n_csc_blocks, sys->sums_bwd, s));
   return MC_OK;
 }
 
@@ -1914,8 +1943,8 @@ static int batch_segments(const uint32_t *ptr, int64_t n, int64_t nnz, const uin
   warp = 0;
   if (cnt == 0) return MC_OK;
   if ((double)nnz / (double)cnt < 16.0) return MC_OK;  // warp chunks: units set by batch_create
-  bool w = false;
-  MCS_TRY(stream_tiles(cptr, cnt, nnz, tiles, n_tiles, w, s, true));
+  int sums = kChunks;
+  MCS_TRY(stream_tiles(cptr, cnt, nnz, tiles, n_tiles, sums, s, true));
   warp = 1;
   return MC_OK;
 }
