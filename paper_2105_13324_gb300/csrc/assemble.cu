@@ -721,6 +721,46 @@ static int assemble_buckets(mc_system *sys, const uint64_t *keys, int64_t n, cud
   return MC_OK;
 }
 
+// The CSR of the nu > 0 entries whose keys (j << b) | v, b = bits of N - 1, stand
+// in CSC order: sorted with the counts `cnt` (or, weighted, the CSC position of
+// each entry, whose weight and count `went` holds) as payload, then columns and
+// row_ptr (allocated by the caller) in sorted order.  tkeys and cnt are used up.
+static int csr_by_radix(mc_system *sys, DevBuf &tkeys, DevBuf &cnt, DevBuf &went, int64_t nu, cudaStream_t s) {
+  const int64_t M = sys->n_rows;
+  const int b = bits_for((uint64_t)sys->n_cols - 1);
+  DevBuf tkeys_alt, tcnt_alt, tperm;
+  MCS_TRY(sys->col_idx.alloc((size_t)nu * sizeof(uint32_t), s));
+  MCS_TRY(sys->csr_cnt.alloc((size_t)nu * sizeof(uint32_t), s));
+  MCS_TRY(tkeys_alt.alloc((size_t)nu * sizeof(uint64_t), s));
+  MCS_TRY(tcnt_alt.alloc((size_t)nu * sizeof(uint32_t), s));
+  if (sys->weighted) {
+    MCS_TRY(tperm.alloc((size_t)nu * sizeof(uint32_t), s));
+    count_launch(); iota_kernel<<<grid_for(nu), 256, 0, s>>>(tperm.as<uint32_t>(), nu);
+    MCS_LAUNCHED();
+  }
+  uint32_t *payload = sys->weighted ? tperm.as<uint32_t>() : cnt.as<uint32_t>();
+  bool talt = false;
+  // the entries are in (v, j) order: a stable sort on the j bits of
+  // (j << b) | v alone gives (j, v) order
+  MCS_TRY(radix_sort_u64(tkeys.as<uint64_t>(), tkeys_alt.as<uint64_t>(), payload, tcnt_alt.as<uint32_t>(), nu,
+                         b + bits_for((uint64_t)M - 1), &talt, s, b));
+  const uint64_t *tk = talt ? tkeys_alt.as<uint64_t>() : tkeys.as<uint64_t>();
+  const uint32_t *tc = talt ? tcnt_alt.as<uint32_t>() : payload;
+  count_launch();
+  csr_split_kernel<<<grid_for(nu), 256, 0, s>>>(tk, nu, b, sys->col_idx.as<uint32_t>(), sys->row_ptr.as<uint32_t>(), M);
+  MCS_LAUNCHED();
+  if (sys->weighted) {
+    MCS_TRY(sys->csr_wq.alloc((size_t)nu * sizeof(uint64_t), s));
+    count_launch();
+    gather_entries_kernel<<<grid_for(nu), 256, 0, s>>>(tc, nu, went.as<WEntry>(), sys->csr_cnt.as<uint32_t>(),
+                                                       sys->csr_wq.as<uint64_t>());
+    MCS_LAUNCHED();
+  } else {
+    MCS_CUDA(cudaMemcpyAsync(sys->csr_cnt.p, tc, (size_t)nu * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+  }
+  return MC_OK;
+}
+
 // ---------------------------------------------------------------------------
 // assembly by sorted segments (weighted events, and columns or rows too long
 // for the buckets above)
@@ -1026,6 +1066,28 @@ __global__ void __launch_bounds__(kSegThreads) segment_transpose_kernel(const ui
   }
 }
 
+// CSC entries as keys (j << b) | v in CSC order, weighted with their weight and
+// count side by side, for csr_by_radix.
+template <bool W>
+__global__ void __launch_bounds__(kSegThreads) segment_keys_kernel(const uint32_t *col_ptr, int64_t n_cols,
+                                                                const uint32_t *row_idx, const uint32_t *cnt,
+                                                                const uint64_t *wq, int b, uint64_t *tkeys,
+                                                                WEntry *ent) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n_warps = ((int64_t)gridDim.x * kSegThreads) >> 5;
+  for (int64_t c = ((int64_t)blockIdx.x * kSegThreads + threadIdx.x) >> 5; c < n_cols; c += n_warps) {
+    const uint32_t e = col_ptr[c + 1];
+    for (uint32_t k = col_ptr[c] + lane; k < e; k += 32) {
+      tkeys[k] = ((uint64_t)row_idx[k] << b) | (uint64_t)c;
+      if constexpr (W) {
+        WEntry x;
+        x.w = wq[k]; x.cnt = cnt[k]; x.pad = 0u;
+        ent[k] = x;
+      }
+    }
+  }
+}
+
 // The same in two passes, for matrices beyond the L2.  Pass 1 sorts tiles of
 // CSC entries by block of 2^shift rows in shared memory and appends each run
 // to its row block's part of the CSR range; in pass 2 one thread block takes a
@@ -1199,15 +1261,16 @@ static int launch_segments(Kernel *k, size_t key_bytes, int maxk, int64_t n_seg,
 
 // The CSC and CSR of n > 0 events (with the projector values and the column
 // sums) by sorted segments.  Sets *done, or leaves the matrix unfinished (and
-// the events untouched) when a column holds more than kSegLen events or a row
-// more than kSegLen entries; the events' buffers are released once they are
-// not needed.
+// the events untouched) when a column holds more than kSegLen events, which a
+// mean above that shows without counting.  The events' buffers are released
+// once they are not needed.
 template <bool W>
 static int assemble_segments(mc_system *sys, DevBuf &key_buf, DevBuf *weight_buf, int64_t n, cudaStream_t s,
                              bool *done) {
   *done = false;
   const uint64_t *keys = key_buf.as<uint64_t>(), *weights = W ? weight_buf->as<uint64_t>() : nullptr;
   const int64_t M = sys->n_rows, N = sys->n_cols;
+  if (n > kSegLen * N) return MC_OK;
   const Div64 dm = make_div((uint64_t)M);
   DevBuf cnt, start, flag, tmp;
   MCS_TRY(cnt.alloc((size_t)(N + 1) * 4, s));
@@ -1282,7 +1345,28 @@ static int assemble_segments(mc_system *sys, DevBuf &key_buf, DevBuf *weight_buf
   MCS_TRY(sys->row_ptr.alloc((size_t)(M + 1) * 4, s));
   MCS_TRY(exclusive_scan_u32(rhist.as<uint32_t>(), sys->row_ptr.as<uint32_t>(), M + 1, s));
   MCS_TRY(max_of(rhist, M, flag, &longest, s));  // waits, max_count included
-  if (longest > (uint32_t)kSegLen) return MC_OK;
+  sys->nnz = nnz;
+  sys->max_count = max_count;
+  if (longest > (uint32_t)kSegLen) {
+    // rows too long for a warp: the CSC stands, the CSR by radix sort (the
+    // projector values then come from the counts or weights)
+    key_buf.release();
+    if (W) weight_buf->release();
+    sys->csc_val.release();
+    DevBuf tkeys, ucnt, went;
+    MCS_TRY(tkeys.alloc((size_t)nnz * sizeof(uint64_t), s));
+    if (W) {
+      MCS_TRY(went.alloc((size_t)nnz * sizeof(WEntry), s));
+    } else {
+      MCS_TRY(ucnt.alloc((size_t)nnz * 4, s));
+      MCS_CUDA(cudaMemcpyAsync(ucnt.p, csc_cnt, (size_t)nnz * 4, cudaMemcpyDeviceToDevice, s));
+    }
+    MCS_TRY(launch_segments(segment_keys_kernel<W>, 0, 1, N, s, col_ptr, N, row_idx, csc_cnt, csc_wq,
+                            bits_for((uint64_t)N - 1), tkeys.as<uint64_t>(), went.as<WEntry>()));
+    MCS_TRY(csr_by_radix(sys, tkeys, ucnt, went, nnz, s));
+    *done = true;
+    return MC_OK;
+  }
   const uint32_t *row_ptr = sys->row_ptr.as<uint32_t>();
   // the matrix will be finished here: the events are not needed again, and
   // their buffers hold the entries on their way where they are large enough
@@ -1344,8 +1428,6 @@ static int assemble_segments(mc_system *sys, DevBuf &key_buf, DevBuf *weight_buf
     if (longest > 32 * kShortK)
       MCS_TRY(wide ? go(segment_rows_kernel<uint64_t, 32, W>, 8, 32) : go(segment_rows_kernel<uint32_t, 32, W>, 4, 32));
   }
-  sys->nnz = nnz;
-  sys->max_count = max_count;
   sys->values_ready = true;
   *done = true;
   return MC_OK;
@@ -1433,50 +1515,16 @@ static int assemble_radix(mc_system *sys, DevBuf &keys, int64_t n, cudaStream_t 
   }
   ukeys.release();
 
-  // 4. CSR: sort the transposed keys (with the counts, or, weighted, the CSC
-  // position of each entry), then columns and row_ptr in sorted order
-  {
-    MCS_TRY(sys->row_ptr.alloc((M + 1) * sizeof(uint32_t), s));
-    MCS_TRY(sys->col_idx.alloc(nnz_b * sizeof(uint32_t), s));
-    MCS_TRY(sys->csr_cnt.alloc(nnz_b * sizeof(uint32_t), s));
-    if (nu > 0) {
-      DevBuf tkeys_alt, tcnt_alt, tperm;
-      MCS_TRY(tkeys_alt.alloc(nu * sizeof(uint64_t), s));
-      MCS_TRY(tcnt_alt.alloc(nu * sizeof(uint32_t), s));
-      if (weights) {
-        MCS_TRY(tperm.alloc(nu * sizeof(uint32_t), s));
-        count_launch(); iota_kernel<<<grid_for(nu), 256, 0, s>>>(tperm.as<uint32_t>(), nu);
-        MCS_LAUNCHED();
-      }
-      uint32_t *payload = weights ? tperm.as<uint32_t>() : ucnt.as<uint32_t>();
-      bool talt = false;
-      // the entries are in (v, j) order: a stable sort on the j bits of
-      // (j << b) | v alone gives (j, v) order
-      MCS_TRY(radix_sort_u64(tkeys.as<uint64_t>(), tkeys_alt.as<uint64_t>(), payload,
-                             tcnt_alt.as<uint32_t>(), nu, b + bits_for(M - 1), &talt, s, b));
-      const uint64_t *tk = talt ? tkeys_alt.as<uint64_t>() : tkeys.as<uint64_t>();
-      const uint32_t *tc = talt ? tcnt_alt.as<uint32_t>() : payload;
-      count_launch();
-      csr_split_kernel<<<grid_for(nu), 256, 0, s>>>(tk, nu, b, sys->col_idx.as<uint32_t>(),
-                                                    sys->row_ptr.as<uint32_t>(), (int64_t)M);
-      MCS_LAUNCHED();
-      if (weights) {
-        MCS_TRY(sys->csr_wq.alloc(nu * sizeof(uint64_t), s));
-        count_launch();
-        gather_entries_kernel<<<grid_for(nu), 256, 0, s>>>(tc, nu, went.as<WEntry>(), sys->csr_cnt.as<uint32_t>(),
-                                                           sys->csr_wq.as<uint64_t>());
-        MCS_LAUNCHED();
-      } else {
-        MCS_CUDA(cudaMemcpyAsync(sys->csr_cnt.p, tc, nu * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-      }
-    } else {
-      MCS_CUDA(cudaMemsetAsync(sys->row_ptr.p, 0, (M + 1) * sizeof(uint32_t), s));
-      if (weights) MCS_TRY(sys->csr_wq.alloc(sizeof(uint64_t), s));
-    }
+  // 4. CSR
+  MCS_TRY(sys->row_ptr.alloc((M + 1) * sizeof(uint32_t), s));
+  if (nu > 0) {
+    MCS_TRY(csr_by_radix(sys, tkeys, ucnt, went, nu, s));
+  } else {
+    MCS_TRY(sys->col_idx.alloc(sizeof(uint32_t), s));
+    MCS_TRY(sys->csr_cnt.alloc(sizeof(uint32_t), s));
+    MCS_CUDA(cudaMemsetAsync(sys->row_ptr.p, 0, (M + 1) * sizeof(uint32_t), s));
+    if (weights) MCS_TRY(sys->csr_wq.alloc(sizeof(uint64_t), s));
   }
-  tkeys.release();
-  went.release();
-
   return MC_OK;
 }
 
