@@ -1,10 +1,7 @@
 """Build libmcspect.so (the CUDA library behind include/mcspect.h) in-tree.
 
 nvcc compiles each translation unit for sm_103a in parallel, then links a
-shared library into paper_2105_13324_gb300/_build/.  The single-precision
-transport unit flushes denormals (its logarithms, reciprocals and roots then
-need no scaling steps: 40.4 -> 37.9 ms per 1e9 torso histories together with
-wider shared-memory words, the same matrix); the double-precision
+shared library into paper_2105_13324_gb300/_build/.  The double-precision
 transport unit is compiled with --fmad=false (products and sums rounded as
 written).  Host code is compiled with -ffp-contract=off for the same reason.
 """
@@ -24,7 +21,7 @@ UNITS = {
     "api.cu": [],
     "assemble.cu": [],
     "mlem.cu": [],
-    "transport_f32.cu": ["-ftz=true"],
+    "transport_f32.cu": [],
     "transport_f64.cu": ["--fmad=false"],
 }
 

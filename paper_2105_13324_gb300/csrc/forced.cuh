@@ -112,7 +112,7 @@ __device__ __forceinline__ bool make_ray(const TArgs<float> &a, const FdRec<floa
     const float qx = px + t * dx, qy = py + t * dy, qz = pz + t * dz;
     float au = -qx * sk + qy * ck;
     float bv = qz;
-    const float rr = sqrt0<float>(-2.0f * __logf(u2));
+    const float rr = sqrt0<float>(-2.0f * ln_normal(u2));
     float cb, sb;
     cos_sin_2pi<float>(u3, cb, sb);
     au += a.sigma * (rr * cb);
