@@ -86,7 +86,7 @@ def penalised_reconstruct(system, y, shape, beta: float, n_iter: int, alpha: flo
     bp = torch.empty(n, dtype=torch.float32, device=dev)
     gp = torch.empty(n, dtype=torch.float32, device=dev) if beta > 0 else None
     # log-likelihood and prior value side by side: one read (and one wait) per
-    # objective instead of two, 8.6 -> 7.6 ms for 4 iterations at 128^3
+    # objective instead of two, a millisecond of nine for 4 iterations at 128^3
     terms = torch.zeros(2, dtype=torch.float64, device=dev)
     ll, pv = terms[0:1], terms[1:2]
 

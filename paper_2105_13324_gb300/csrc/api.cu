@@ -450,8 +450,7 @@ static int tally_from_plan(mc_plan *pl, uint64_t first, uint64_t count, uint64_t
       return MC_ECUDA;
     }
     {
-      // every history ends in exactly one fate; fewer means a transport
-      // launch gave up (its random-word producer stopped answering)
+      // every history ends in exactly one fate
       const unsigned long long done = hctr[1] + hctr[2] + hctr[3] + hctr[4];
       if (done != count) {
         set_error("transport finished %llu of %llu histories", done, (unsigned long long)count);

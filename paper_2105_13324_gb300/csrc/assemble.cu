@@ -3,11 +3,14 @@
 // are counts of histories).
 //
 // Events arrive as 64-bit keys v*M + j in arbitrary order (the transport
-// kernel appends them with atomics).  A stable LSD radix sort orders them by
-// (v, j); a run-length pass turns runs of equal keys into (v, j, count)
-// triples, which are the CSC form.  The CSR form comes from a second radix
-// sort of the (j*N + v, count) pairs.  Everything is integer work, so the
-// matrix is bit-identical from run to run.  No floating-point atomics.
+// kernel appends them with atomics), weighted ones with a fixed-point weight.
+// Three ways lead to the same CSC and CSR: buckets (a thread per column and per
+// row) for unweighted events in short columns and rows, sorted segments (a warp
+// per column and per row of up to 1024 elements) for weighted events and longer
+// ones, and a stable LSD radix sort by (v, j) with a run-length pass for columns
+// beyond that, which also makes the CSR where rows are.  Everything is integer
+// work, so the matrix is bit-identical from run to run.  No floating-point
+// atomics.
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 
@@ -769,10 +772,11 @@ static int csr_by_radix(mc_system *sys, DevBuf &tkeys, DevBuf &cnt, DevBuf &went
 // sorts each column by row in its registers, counts the distinct rows, and,
 // once the column pointers are known, sorts again and writes the merged
 // entries, their projector values and the column sums.  The CSR is made the
-// same way: entries placed in their rows' segments, a warp per row.  Sorting
-// twice (~2 warp instructions per event) is cheaper than writing the sorted
-// events out and reading them back.  Integer work on whole segments, so the
-// matrix does not depend on the order of arrival.
+// same way: entries placed in their rows' segments, a warp per row (by radix
+// sort where a row has more than kSegLen entries).  Sorting twice (~2 warp
+// instructions per event) is cheaper than writing the sorted events out and
+// reading them back.  Integer work on whole segments, so the matrix does not
+// depend on the order of arrival.
 //
 // Bound by the placement passes (a scattered store per entry, and a returning
 // atomic per run of events of one column) and by memory otherwise: about 110
@@ -1181,7 +1185,8 @@ __global__ void row_block_starts_kernel(const uint32_t *row_ptr, int64_t n_rows,
 
 // Pass 2: row block b = rows [b << shift, (b + 1) << shift), its entries those
 // of its CSR range.  Two blocks of 512 threads per SM: the rows being filled
-// are then ~300 x 2048, whose half-written lines (80 MB) stay in the L2.
+// are then ~300 x 2048, whose half-written lines (80 MB) stay in the L2 (chosen
+// on a matrix of 2.5e8 entries).
 constexpr int kPlaceThreads = 512;
 template <bool W>
 __global__ void __launch_bounds__(kPlaceThreads, 2) place_rows_kernel(const SegEntry<W> *in, const uint32_t *row_ptr,

@@ -19,15 +19,11 @@ namespace mcs {
 //
 // Bound by latency and issue together: each step is one dependent load of the
 // grid (material and distance in one 16-bit word), of which the L1 -- what the
-// stacks leave of it -- holds few lines.  Six blocks an SM (24 warps) leave
-// 100 KB of it and are faster than eight (23.3 against 24.8 ms) or five
-// (24.9).  2^21 histories of the 128^3 torso towards 120 views (3.9e8 copies,
-// 2.6e8 events): 32.6 -> 23.3 ms, the same events.  On the way: rays on a stack
-// but an atomic and an FP64 conversion per hand-out 29 to 38 ms (a warp waits
-// for every append; FP64 instructions cost the same for 6 lanes as for 32);
-// events appended a warp at a time, weights converted from the float 28.9 ms;
-// no step counter, clamps for compares, two steps a vote, 80-byte rays 23.3 ms.
-// Rays of unequal length handed out when 8 lanes are idle: 4 to 16 within 2 %.
+// stacks leave of it -- holds few lines.  The launch takes what an SM holds:
+// seven blocks at 68 registers (six run alike, eight are 5 % slower, five 7 %).
+// 2^21 histories of the 128^3 torso towards 120 views (3.9e8 copies, 2.6e8
+// events): 24 ms, 33 with a lane per copy to its end; the same events.  Rays of
+// unequal length are handed out when 8 lanes are idle: 4 to 16 within 2 %.
 constexpr int kRayThreads = 128;
 constexpr int kRayPool = 64;   // rays waiting per warp: 31 before a round of 32 at most
 constexpr int kRayQuads = 5;   // 16-byte words per ray

@@ -35,13 +35,9 @@ namespace mcs {
 // flight round generates the next block once for both flights.
 //
 // Bound by instruction issue (75 % of the issue slots).  10^9 histories of the
-// 128^3 torso: 32.7 ms, 31 warp instructions per history at 27 of 32 lanes;
-// the former kernel (one history per lane, lanes waiting for 8 to 12 others at
-// the same step) took 81.4 ms, 71 instructions at 13 lanes, with the same
-// matrix and fates.  On the way: stacks with scalar words and branching
-// flights 40.4 ms, 16-byte words and flushed denormals 37.9 ms, flights
-// without branches and unfinished scatters put back after two blocks of
-// trials 32.7 ms.
+// 128^3 torso: 33.0 ms, 31 warp instructions per history at 27 of 32 lanes; one
+// history per lane, lanes waiting for 8 to 12 others at the same step, took
+// 81.4 ms, 71 instructions at 13 lanes, with the same matrix and fates.
 //
 // A warp holds at most 94 photons, so kPool slots suffice: an emission round
 // starts with at most 31 photons at a collision, fewer photons ready to fly

@@ -614,9 +614,10 @@ __global__ void __launch_bounds__(kStreamThreads) stream_back_kernel(const uint3
 // block.
 constexpr int kChunkWindow = 128;
 constexpr int kChunkThreads = 128;
-// The batch kernels' window with four rows a lane: rows of 1.1 entries make
-// chunks of ~140 entries, one window of 160 where 128 takes two, the second
-// nearly empty: 64 mixed systems, 30 iterations, 3.47 -> 3.22 ms (192 entries
+// The batch kernels' window with four rows a lane.  Four rows a lane are taken
+// up to 1.5 entries a row; those of serving systems, 1.1, make chunks of ~140
+// entries, one window of 160 where 128 takes two, the second nearly empty (from
+// 1.25 on there are two again, as with 128): 64 mixed systems, 30 iterations, 3.47 -> 3.22 ms (192 entries
 // 3.51, 256 3.59: registers), and 3.16 with the smaller shared memory of
 // batches without tiles.  One and two rows a lane keep the 128 (chunks of ~35
 // entries gain nothing, and a batch of one takes 0.222 instead of 0.233 ms at
